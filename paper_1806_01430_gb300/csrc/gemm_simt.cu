@@ -1,152 +1,309 @@
 // FP32 SIMT GEMM on the CUDA cores: C = alpha * A @ B + beta * C0.
 //
-// The "plain FP32" comparison path.  128 x 128 block tile, K step 16, 256 threads,
-// each thread an 8 x 8 register tile (two 4-row by two 4-column quadrants so that
-// shared-memory reads are 16-byte and conflict-free), shared memory double buffered
-// with one barrier per K step.  Accuracy: a single binary32 accumulator over a long
-// K grows its rounding error with K, so the K loop is split into chunks of `kchunk`
-// elements; each chunk is summed from zero in registers and then added into a
-// shared-memory tile of running sums (element-major, so every access is conflict-free),
-// which keeps the registers under 128 for two blocks per SM.  A and B are row-major
-// (A: M x K, B: K x N).
+// The "plain FP32" path; A and B are row-major (A: M x K, B: K x N).
+//
+// Accuracy: a single binary32 accumulator over a long K grows its rounding error with K, so
+// the K loop is split into chunks of `kchunk` elements; each chunk is summed from zero in
+// registers and the chunk sums are then added in order.  Every element takes the same
+// operations in the same order whatever the tile and the split, and as the host loop does, so
+// all give the same bits.
+//
+// What bounds it: the FP32 lanes (128 multiply-adds per clock and SM) and, next to them, shared
+// memory, which returns 128 bytes per clock and SM: with an 8 x 8 register tile per thread the
+// operand reads take as many clocks as the multiply-adds (that kernel reached 0.61 of the
+// lanes), with 8 x 16 three quarters of them.  Packed multiply-adds (fma.rn.f32x2: two columns
+// of a row, the same rounding per element) leave the issue slots that the loads, the operand
+// duplication and the loop need.  Both operands go to shared memory by cp.async (no register
+// staging): A as rows of BK elements (a thread reads four k of a row at once), B as it lies.
+// A small problem has too few tiles to fill the GPU; since the chunks are summed apart anyway, a
+// cluster can split them (no order changes), and smaller tiles serve where that is not enough.
+// Measured, n x n x n, us (before: 128 x 128 tiles of 8 x 8 per thread, scalar FFMAs):
+//   n = 256: 40.8 -> 9.5, 1000: 148 -> 58, 1001: 158 -> 77, 2048: 431 -> 347, 4096: 3020 -> 2500
+//   (55 of 80 TFLOP/s).  What is left: two warps per scheduler issue a packed multiply-add every
+//   other clock with little to cover the operand reads, and the last wave of tiles.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "gao_internal.h"
 
 namespace gao {
 namespace {
 
-constexpr int BM = 128, BN = 128, BK = 16;
-constexpr int kThreads = 256;
-constexpr size_t kTileFloats = 2 * (size_t)BK * (BM + BN);       // double-buffered A and B tiles
-constexpr size_t kSmemBytes = (kTileFloats + 64 * kThreads) * 4;  // + the chunk-sum tile
+// TM x TN elements per thread; a warp is 4 x 8 threads; WM x WN warps form the block tile.
+template <int TM_, int TN_, int WM_, int WN_, int BK_, int STAGES_, int MINB_>
+struct Shape {
+    static constexpr int TM = TM_, TN = TN_, WM = WM_, WN = WN_, BK = BK_, STAGES = STAGES_, MINB = MINB_;
+    static constexpr int THREADS = 32 * WM * WN;
+    static constexpr int BM = WM * 4 * TM, BN = WN * 8 * TN;
+    static constexpr int LDA = BK + 4;  // rows of A 16 bytes apart in banks: four rows read at once without conflicts
+    static constexpr int A_FLOATS = BM * LDA, B_FLOATS = BK * BN;  // one stage
+    static constexpr int E = TM * TN / 4;                          // groups of four columns per thread
+    static constexpr size_t TILE_BYTES = (size_t)STAGES * (A_FLOATS + B_FLOATS) * 4;
+    static constexpr size_t SUM_BYTES = (size_t)E * THREADS * 16;  // running sums, or a split chunk's sums
+};
+using Large = Shape<8, 16, 4, 1, 16, 2, 2>;   // 128 x 128, 128 threads
+using Medium = Shape<8, 8, 2, 1, 16, 3, 4>;   // 64 x 64, 64 threads
+using Small = Shape<4, 4, 2, 1, 32, 4, 4>;    // 32 x 32, 64 threads
 
-template <bool VEC>
-__global__ void __launch_bounds__(kThreads, 2)
-    sgemm_kernel(float* C, const float* __restrict__ A, const float* __restrict__ B,
-                 const float* C0, int64_t M, int64_t N, int64_t K, float alpha, float beta, int64_t kc) {
+using f32x2 = unsigned long long;  // two binary32 values, the lower address in the low half
+
+// acc = a * b + acc in both halves, one rounding each.
+__device__ __forceinline__ void ffma2(f32x2& acc, f32x2 a, f32x2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 unpack(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 dup(float a) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
+}
+// BYTES from global to shared memory without passing through registers; zeros where !in.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint32_t dst, const float* src, bool in) {
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+
+// va, vb, vc: rows of A; of B; of C and C0 are 16-byte aligned.  SPLIT: a cluster of
+// ceil(K / kc) blocks along z shares a tile, each summing one chunk; the sums meet in shared
+// memory and each block adds, in chunk order, and stores its share of the tile.
+template <class S, bool SPLIT>
+__global__ void __launch_bounds__(S::THREADS, S::MINB)
+    sgemm_kernel(float* C, const float* __restrict__ A, const float* __restrict__ B, const float* C0, int64_t M,
+                 int64_t N, int64_t K, float alpha, float beta, int64_t kc, bool va, bool vb, bool vc) {
+    constexpr int TM = S::TM, TN = S::TN, BK = S::BK, THREADS = S::THREADS;
     extern __shared__ __align__(16) float smem[];
-    float* As = smem;                       // [2][BK][BM]
-    float* Bs = smem + 2 * BK * BM;         // [2][BK][BN]
-    float* sum = smem + kTileFloats;        // [64][kThreads]: element-major, conflict-free
-    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-    const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
+    float* As = smem;                                        // [STAGES][BM][LDA]
+    float* Bs = smem + S::STAGES * S::A_FLOATS;              // [STAGES][BK][BN]
+    float4* ssum = reinterpret_cast<float4*>(smem + S::STAGES * (S::A_FLOATS + S::B_FLOATS));  // [E][THREADS]
+    const uint32_t as_addr = (uint32_t)__cvta_generic_to_shared(As);
+    const uint32_t bs_addr = (uint32_t)__cvta_generic_to_shared(Bs);
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int wm = w / S::WN, wn = w % S::WN, ty = lane >> 3, tx = lane & 7;
+    const int64_t m0 = (int64_t)blockIdx.y * S::BM, n0 = (int64_t)blockIdx.x * S::BN;
+    // this block's part of K: everything, or one chunk
+    const int64_t kbeg = SPLIT ? (int64_t)blockIdx.z * kc : 0;
+    const int64_t kend = SPLIT && kbeg + kc < K ? kbeg + kc : K;
+    const int64_t nk = (kend - kbeg + BK - 1) / BK;
+    const bool one = SPLIT || K <= kc;  // a single chunk: its sums are not added to anything here
 
-    // global -> register staging: A row am, k offsets ak..ak+7; B rows bk and bk+8,
-    // columns bn..bn+3
-    const int am = t >> 1, ak = (t & 1) * 8;
-    const int bk = t >> 5, bn = (t & 31) * 4;
-    float ra[8], rb[8];
-
-    auto load = [&](int64_t k0) {
-        const int64_t gm = m0 + am;
+    auto load = [&](int64_t kt) {
+        const int st = (int)(kt % S::STAGES);
+        const int64_t k0 = kbeg + kt * BK;
+        const uint32_t a_dst = as_addr + (uint32_t)(st * S::A_FLOATS) * 4, b_dst = bs_addr + (uint32_t)(st * S::B_FLOATS) * 4;
+        if (va) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int64_t gk = k0 + ak + 4 * h;
-            if (VEC) {
-                float4 v = make_float4(0, 0, 0, 0);
-                if (gm < M && gk < K) v = *reinterpret_cast<const float4*>(A + gm * K + gk);
-                ra[4 * h] = v.x, ra[4 * h + 1] = v.y, ra[4 * h + 2] = v.z, ra[4 * h + 3] = v.w;
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) ra[4 * h + q] = (gm < M && gk + q < K) ? A[gm * K + gk + q] : 0.0f;
+            for (int i = 0; i < S::BM * BK / 4 / THREADS; ++i) {
+                const int e = i * THREADS + t, r = e / (BK / 4), c = e % (BK / 4) * 4;
+                const bool in = m0 + r < M && k0 + c < kend;
+                cp_async<16>(a_dst + (uint32_t)(r * S::LDA + c) * 4, in ? A + (m0 + r) * K + k0 + c : A, in);
             }
-            const int64_t gkb = k0 + bk + 8 * h, gn = n0 + bn;
-            if (VEC) {
-                float4 v = make_float4(0, 0, 0, 0);
-                if (gkb < K && gn < N) v = *reinterpret_cast<const float4*>(B + gkb * N + gn);
-                rb[4 * h] = v.x, rb[4 * h + 1] = v.y, rb[4 * h + 2] = v.z, rb[4 * h + 3] = v.w;
-            } else {
+        } else {
+#pragma unroll 4
+            for (int i = 0; i < S::BM * BK / THREADS; ++i) {
+                const int e = i * THREADS + t, r = e / BK, c = e % BK;
+                const bool in = m0 + r < M && k0 + c < kend;
+                cp_async<4>(a_dst + (uint32_t)(r * S::LDA + c) * 4, in ? A + (m0 + r) * K + k0 + c : A, in);
+            }
+        }
+        if (vb) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) rb[4 * h + q] = (gkb < K && gn + q < N) ? B[gkb * N + gn + q] : 0.0f;
+            for (int i = 0; i < BK * S::BN / 4 / THREADS; ++i) {
+                const int e = i * THREADS + t, r = e / (S::BN / 4), c = e % (S::BN / 4) * 4;
+                const bool in = k0 + r < kend && n0 + c < N;
+                cp_async<16>(b_dst + (uint32_t)(r * S::BN + c) * 4, in ? B + (k0 + r) * N + n0 + c : B, in);
+            }
+        } else {
+#pragma unroll 4
+            for (int i = 0; i < BK * S::BN / THREADS; ++i) {
+                const int e = i * THREADS + t, r = e / S::BN, c = e % S::BN;
+                const bool in = k0 + r < kend && n0 + c < N;
+                cp_async<4>(b_dst + (uint32_t)(r * S::BN + c) * 4, in ? B + (k0 + r) * N + n0 + c : B, in);
             }
         }
     };
-    auto store = [&](int buf) {
-        float* as = As + buf * BK * BM;
-        float* bs = Bs + buf * BK * BN;
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+
+    f32x2 acc[TM][TN / 2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) as[(ak + q) * BM + am] = ra[q];
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-            *reinterpret_cast<float4*>(bs + (bk + 8 * h) * BN + bn) =
-                make_float4(rb[4 * h], rb[4 * h + 1], rb[4 * h + 2], rb[4 * h + 3]);
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+    // group e = (row i, column quad h) of this thread's sums
+    auto group = [&](int i, int h) {
+        const float2 u = unpack(acc[i][2 * h]), v = unpack(acc[i][2 * h + 1]);
+        return make_float4(u.x, u.y, v.x, v.y);
     };
-
-    float acc[8][8];
+    if (!one) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-#pragma unroll
-    for (int e = 0; e < 64; ++e) sum[e * kThreads + t] = 0.0f;
-
-    const int64_t nk = (K + BK - 1) / BK;
-    if (nk > 0) {
-        load(0);
-        store(0);
+        for (int e = 0; e < S::E; ++e) ssum[e * THREADS + t] = make_float4(0, 0, 0, 0);
     }
-    __syncthreads();
+
+#pragma unroll
+    for (int s = 0; s < S::STAGES - 1; ++s) {
+        if (s < nk) load(s);
+        commit();
+    }
+    const int64_t chunk_tiles16 = kc / 16;  // 16-element steps per chunk
+    int64_t left = chunk_tiles16;
     for (int64_t kt = 0; kt < nk; ++kt) {
-        const int buf = (int)(kt & 1);
-        if (kt + 1 < nk) load((kt + 1) * BK);
-        const float* as = As + buf * BK * BM;
-        const float* bs = Bs + buf * BK * BN;
+        asm volatile("cp.async.wait_group %0;" ::"n"(S::STAGES - 2) : "memory");
+        __syncthreads();  // stage kt has landed for every thread; everyone is done with stage kt - 1
+        if (kt + S::STAGES - 1 < nk) load(kt + S::STAGES - 1);
+        commit();
+        const int st = (int)(kt % S::STAGES);
+        const float* as = As + st * S::A_FLOATS + (wm * 4 * TM + ty) * S::LDA;  // rows ty, ty + 4, ...
+        const float* bs = Bs + st * S::B_FLOATS + wn * 8 * TN + tx * 4;         // column quads 32 apart
+#pragma unroll 1
+        for (int g = 0; g < BK / 16; ++g) {  // 16 elements of K
+            // fragments one step ahead of their use: B's of the next k, A's of the next pair of k
+            float2 fa[2][TM];
+            f32x2 fb[2][TN / 2];
+            auto load_a = [&](int k2, float2 (&d)[TM]) {
 #pragma unroll
-        for (int k = 0; k < BK; ++k) {
-            const float4 a0 = *reinterpret_cast<const float4*>(as + k * BM + ty * 4);
-            const float4 a1 = *reinterpret_cast<const float4*>(as + k * BM + 64 + ty * 4);
-            const float4 b0 = *reinterpret_cast<const float4*>(bs + k * BN + tx * 4);
-            const float4 b1 = *reinterpret_cast<const float4*>(bs + k * BN + 64 + tx * 4);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                for (int i = 0; i < TM; ++i)
+                    d[i] = *reinterpret_cast<const float2*>(as + i * 4 * S::LDA + g * 16 + 2 * k2);
+            };
+            auto load_b = [&](int k, f32x2 (&d)[TN / 2]) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        if (kt + 1 < nk) store(buf ^ 1);
-        __syncthreads();
-        if (((kt + 1) * BK) % kc == 0 || kt + 1 == nk) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) sum[(i * 8 + j) * kThreads + t] += acc[i][j], acc[i][j] = 0.0f;
-        }
-    }
-
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int64_t gm = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-        if (gm >= M) continue;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int64_t gn = n0 + h * 64 + tx * 4;
-            float r[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) r[q] = alpha * sum[(i * 8 + h * 4 + q) * kThreads + t];
-            if (VEC && gn + 3 < N) {
-                if (beta != 0.0f) {
-                    const float4 c = *reinterpret_cast<const float4*>(C0 + gm * N + gn);
-                    r[0] = fmaf(beta, c.x, r[0]);
-                    r[1] = fmaf(beta, c.y, r[1]);
-                    r[2] = fmaf(beta, c.z, r[2]);
-                    r[3] = fmaf(beta, c.w, r[3]);
+                for (int h = 0; h < TN / 4; ++h) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(bs + (g * 16 + k) * S::BN + h * 32);
+                    d[2 * h] = v.x;
+                    d[2 * h + 1] = v.y;
                 }
-                *reinterpret_cast<float4*>(C + gm * N + gn) = make_float4(r[0], r[1], r[2], r[3]);
-            } else {
+            };
+            load_a(0, fa[0]);
+            load_b(0, fb[0]);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (gn + q < N) {
-                        float v = r[q];
-                        if (beta != 0.0f) v = fmaf(beta, C0[gm * N + gn + q], v);
-                        C[gm * N + gn + q] = v;
-                    }
+            for (int k = 0; k < 16; ++k) {
+                if (k + 1 < 16) load_b(k + 1, fb[(k + 1) & 1]);
+                if (k % 2 == 0 && k + 2 < 16) load_a(k / 2 + 1, fa[(k / 2 + 1) & 1]);
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const float2 v = fa[(k / 2) & 1][i];
+                    const f32x2 aa = dup(k % 2 ? v.y : v.x);
+#pragma unroll
+                    for (int j = 0; j < TN / 2; ++j) ffma2(acc[i][j], aa, fb[k & 1][j]);
+                }
+            }
+            if (!one) {
+                // a chunk (a multiple of 16 elements) is complete, or K is (steps past K hold
+                // zeros and change nothing)
+                left -= 1;
+                if (left == 0 || (kt + 1 == nk && g + 1 == BK / 16)) {
+                    left = chunk_tiles16;
+#pragma unroll
+                    for (int i = 0; i < TM; ++i)
+#pragma unroll
+                        for (int h = 0; h < TN / 4; ++h) {
+                            const float4 v = group(i, h);
+                            float4& s = ssum[(i * (TN / 4) + h) * THREADS + t];
+                            float4 x = s;
+                            x.x += v.x, x.y += v.y, x.z += v.z, x.w += v.w;
+                            s = x;
+                            acc[i][2 * h] = acc[i][2 * h + 1] = 0ull;
+                        }
                 }
             }
         }
     }
+
+    // group e of thread t: alpha times its sums, plus beta C0, stored
+    auto finish = [&](int e, float4 s) {
+        const int i = e / (TN / 4), h = e % (TN / 4);
+        const int64_t gm = m0 + wm * 4 * TM + i * 4 + ty, gn = n0 + wn * 8 * TN + h * 32 + tx * 4;
+        if (gm >= M) return;
+        float r[4] = {alpha * s.x, alpha * s.y, alpha * s.z, alpha * s.w};
+        if (vc) {
+            if (gn >= N) return;
+            if (beta != 0.0f) {
+                const float4 c = *reinterpret_cast<const float4*>(C0 + gm * N + gn);
+                r[0] = fmaf(beta, c.x, r[0]);
+                r[1] = fmaf(beta, c.y, r[1]);
+                r[2] = fmaf(beta, c.z, r[2]);
+                r[3] = fmaf(beta, c.w, r[3]);
+            }
+            *reinterpret_cast<float4*>(C + gm * N + gn) = make_float4(r[0], r[1], r[2], r[3]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (gn + q >= N) continue;
+                float v = r[q];
+                if (beta != 0.0f) v = fmaf(beta, C0[gm * N + gn + q], v);
+                C[gm * N + gn + q] = v;
+            }
+        }
+    };
+    if constexpr (SPLIT) {
+        namespace cg = cooperative_groups;
+        cg::cluster_group cluster = cg::this_cluster();
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int h = 0; h < TN / 4; ++h) ssum[(i * (TN / 4) + h) * THREADS + t] = group(i, h);
+        cluster.sync();
+        const int nb = (int)gridDim.z, rank = (int)blockIdx.z;
+        for (int e = rank; e < S::E; e += nb) {
+            float4 x = make_float4(0, 0, 0, 0);
+            for (int j = 0; j < nb; ++j) {
+                const float4 v = *cluster.map_shared_rank(&ssum[e * THREADS + t], j);
+                x.x += v.x, x.y += v.y, x.z += v.z, x.w += v.w;
+            }
+            finish(e, x);
+        }
+        cluster.sync();  // no block leaves while another still reads its sums
+    } else {
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int h = 0; h < TN / 4; ++h) {
+                const int e = i * (TN / 4) + h;
+                if (one) {  // + 0: the sums start at +0
+                    const float4 v = group(i, h);
+                    finish(e, make_float4(0.0f + v.x, 0.0f + v.y, 0.0f + v.z, 0.0f + v.w));
+                } else {
+                    finish(e, ssum[e * THREADS + t]);
+                }
+            }
+    }
+}
+
+template <class S, bool SPLIT>
+cudaError_t launch_shape(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N, int64_t K,
+                         float alpha, float beta, int64_t kc, cudaStream_t st) {
+    auto kern = sgemm_kernel<S, SPLIT>;
+    constexpr int most = (int)(S::TILE_BYTES + S::SUM_BYTES);
+    static bool attr_set = false;  // per instantiation
+    if (!attr_set) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    auto al = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
+    const bool va = K % 4 == 0 && al(A), vb = N % 4 == 0 && al(B), vc = N % 4 == 0 && al(C) && al(C0);
+    const unsigned nb = SPLIT ? (unsigned)((K + kc - 1) / kc) : 1u;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)((N + S::BN - 1) / S::BN), (unsigned)((M + S::BM - 1) / S::BM), nb);
+    lc.blockDim = dim3(S::THREADS);
+    lc.dynamicSmemBytes = S::TILE_BYTES + (SPLIT || K > kc ? S::SUM_BYTES : 0);
+    lc.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 1;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = nb;
+    lc.attrs = &at;
+    lc.numAttrs = SPLIT ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, kern, C, A, B, C0, M, N, K, alpha, beta, kc, va, vb, vc);
 }
 
 }  // namespace
@@ -154,26 +311,48 @@ __global__ void __launch_bounds__(kThreads, 2)
 cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N,
                              int64_t K, float alpha, float beta, int kchunk, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    int64_t kc = kchunk > 0 ? ((kchunk + BK - 1) / BK) * BK : (int64_t)1 << 62;
-    dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
-    if (grid.y > 65535u) return cudaErrorInvalidValue;
-    const bool vec = (K % 4 == 0) && (N % 4 == 0) &&
-                     ((((uintptr_t)A) | ((uintptr_t)B) | ((uintptr_t)C) | ((uintptr_t)C0)) & 15u) == 0;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(sgemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sgemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
+    if ((M + 127) / 128 > 65535) return cudaErrorInvalidValue;
+    const int64_t kc = kchunk > 0 ? (((int64_t)kchunk + 15) / 16) * 16 : (int64_t)1 << 40;  // above any K: one chunk
+    // The shape, and whether a cluster splits the chunks (2 to 8 of them), with the least
+    // estimated time: the fullest SM holds u blocks, which take max(lat, u w) clocks per element
+    // of K (lat: a block alone, bound by latency; w: its share of a busy SM), plus a fixed cost
+    // (launch, first loads, a split's exchange).  The figures are fits to times measured over
+    // n = 128 .. 4096 (within 10 %); rows that cp.async takes a word at a time cost `ragged` more.
+    struct Model {
+        int tile;
+        double lat, w, fixed, fixed_split, ragged;
+    };
+    static constexpr Model kModel[3] = {{128, 218, 185, 6e3, 20e3, 1.36},
+                                        {64, 140, 55, 6e3, 11e3, 1.53},
+                                        {32, 58, 19, 6e3, 9e3, 1.7}};
+    const bool rows16 = K % 4 == 0 && N % 4 == 0 && ((((uintptr_t)A) | ((uintptr_t)B)) & 15u) == 0;
+    const int64_t chunks = (K + kc - 1) / kc;
+    int best = 0;
+    double least = 0.0;
+    for (int i = 0; i < 6; ++i) {
+        const Model& m = kModel[i >> 1];
+        const bool split = i & 1;
+        const int64_t tm = (M + m.tile - 1) / m.tile, tn = (N + m.tile - 1) / m.tile;
+        if (tm > 65535 || (split && (chunks < 2 || chunks > 8))) continue;
+        const int64_t blocks = tm * tn * (split ? chunks : 1);
+        const double u = (double)((blocks + sm_count() - 1) / sm_count());
+        const double per_k = std::max(m.lat, u * m.w) * (rows16 ? 1.0 : m.ragged);
+        const double cost = per_k * (double)(split ? kc : K) + (split ? m.fixed_split : m.fixed);
+        if (i == 0 || cost < least) {
+            least = cost;
+            best = i;
+        }
     }
-    if (vec)
-        sgemm_kernel<true><<<grid, kThreads, kSmemBytes, st>>>(C, A, B, C0, M, N, K, alpha, beta, kc);
-    else
-        sgemm_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(C, A, B, C0, M, N, K, alpha, beta, kc);
-    return cudaGetLastError();
+#define GAO_SIMT(S, SPLIT) launch_shape<S, SPLIT>(C, A, B, C0, M, N, K, alpha, beta, kc, st)
+    switch (best) {
+        case 0: return GAO_SIMT(Large, false);
+        case 1: return GAO_SIMT(Large, true);
+        case 2: return GAO_SIMT(Medium, false);
+        case 3: return GAO_SIMT(Medium, true);
+        case 4: return GAO_SIMT(Small, false);
+        default: return GAO_SIMT(Small, true);
+    }
+#undef GAO_SIMT
 }
 
 }  // namespace gao
