@@ -518,14 +518,15 @@ gao_status gao_selftest_device_wait(double limit_s, void *stream);
  * GPU's memory, or a latency-critical loop that cannot afford cudaMalloc/cudaFree
  * (which may synchronise the device and can fail with out-of-memory mid-run).
  *
- * It allocates nothing and calls no allocating routine.  Its scratch, one 32-bit key
- * per column, is a fixed array of GAO_COLMAX_NOALLOC_MAX_COLS keys (256 KiB) inside
+ * It allocates nothing and calls no allocating routine.  One kernel forms the maxima
+ * in shared memory; tall inputs of few columns need scratch, one 32-bit key per column,
+ * a fixed array of GAO_COLMAX_NOALLOC_MAX_COLS keys (256 KiB) inside
  * the library; every GPU that loads the library holds that array until the process
  * exits.  cols above the maximum is rejected with GAO_EINVAL.  The first call on a
  * device (with that device current) looks up the array's device address; make that
- * first call before any stream capture.  Every call clears the keys it uses on
+ * first call before any stream capture.  A call that uses the keys clears them on
  * `stream` before reducing, and all calls share the one array: calls whose work
- * overlaps on the GPU (different streams, or several host threads) race and give
+ * overlaps on the GPU (different streams, or several host threads) may race and give
  * wrong results.  Asynchronous on `stream` (NULL: the legacy default stream);
  * dev_in and dev_out are owned by the caller. */
 #define GAO_COLMAX_NOALLOC_MAX_COLS 65536

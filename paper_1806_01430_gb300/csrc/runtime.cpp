@@ -738,8 +738,9 @@ gao_status run_gpu_loop(RunCtx& R, int li) {
         }
         case GAO_LOOP_COLMAX: {
             const gao_buffer& X = shp(L.ins[0]);
-            e = launch_colmax(dptr(L.outs[0]), dptr(L.ins[0]), X.rows, X.cols, (uint32_t*)(a + p->lay.keys_off), st);
-            nl += (X.cols > 0) * (1 + (X.rows > 0));
+            int l = 0;
+            e = launch_colmax(dptr(L.outs[0]), dptr(L.ins[0]), X.rows, X.cols, (uint32_t*)(a + p->lay.keys_off), st, &l);
+            nl += l;
             break;
         }
         case GAO_LOOP_STENCIL3: {
