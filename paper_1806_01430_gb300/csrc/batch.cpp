@@ -377,7 +377,9 @@ gao_status size_tables(gao_batch* b, int reps) {
 gao_status grouped_launch(gao_batch* b, const std::vector<int>& parts, const std::vector<ChainVar*>& cv, bool spans) {
     GAO_CUDA_TRY(cudaEventSynchronize(b->tab_ev));  // the previous table copy has read h_table
     int k = 0, start = 0;
+    bool chain = false;
     for (int r : parts) {
+        chain |= cv[(size_t)r] != nullptr;
         const std::vector<TcProblem>& src = cv[(size_t)r] ? cv[(size_t)r]->probs : b->reps[(size_t)r].probs;
         for (const TcProblem& pr : src) {
             if (k >= b->table_cap) return fail(GAO_EINVAL, "batch problem table overflow");
@@ -396,7 +398,7 @@ gao_status grouped_launch(gao_batch* b, const std::vector<int>& parts, const std
         GAO_CUDA_TRY(cudaMemsetAsync(b->d_span + b->table_cap, 0, sizeof(unsigned long long) * (size_t)k, b->st));
     }
     GAO_CUDA_TRY(cudaEventRecord(b->g0, b->st));
-    GAO_CUDA_TRY(tc_launch_grouped(b->prec, b->chunked, b->d_probs, k, start, b->d_err, b->st));
+    GAO_CUDA_TRY(tc_launch_grouped(b->prec, b->chunked, chain, b->d_probs, k, start, b->d_err, b->st));
     GAO_CUDA_TRY(cudaEventRecord(b->g1, b->st));
     if (spans) {
         GAO_CUDA_TRY(cudaMemcpyAsync(b->h_span, b->d_span, sizeof(unsigned long long) * (size_t)k,
@@ -728,8 +730,9 @@ extern "C" gao_status batch_create(gao_prog* const* progs, int n_progs, gao_batc
     if (b->grouped_gemm) {
         std::string why;
         if (!tc_available(&why)) return bail(fail(GAO_ENODEV, why));
-        if ((e = tc_launch_grouped(b->prec, b->chunked, nullptr, 0, 0, nullptr, b->st)) != cudaSuccess)
-            return bail(cuda_fail(e, "grouped GEMM set-up"));
+        for (bool chain : {false, true})
+            if ((e = tc_launch_grouped(b->prec, b->chunked, chain, nullptr, 0, 0, nullptr, b->st)) != cudaSuccess)
+                return bail(cuda_fail(e, "grouped GEMM set-up"));
         int64_t start = 0;
         for (int i = 0; i < n_progs; ++i) {
             int64_t m, nn, k;

@@ -23,19 +23,20 @@
 // Data flow.  Two memory-bound split kernels write the bfloat16 planes of A
 // (M x K, K contiguous) and of B transposed (N x K, K contiguous), zero-padded to
 // the tile grid.  The MMA kernel is warp-specialised, one 128 x BN output tile per
-// CTA (cta_group::1), 320 threads:
+// CTA (cta_group::1), 320 or 576 threads:
 //   warp 0     TMA producer: cp.async.bulk.tensor 2-D loads of every plane's
 //              128 x 64 (A) and BN x 64 (B) tile into a STAGES-deep ring of
 //              128-byte-swizzled shared-memory stages, completion on mbarriers;
 //   warp 1     allocates tensor memory; one lane issues tcgen05.mma (kind::f16,
 //              M = 128, N = BN, K = 16) for every product and 16-element K step,
 //              and tcgen05.commit releases each stage and each finished accumulator;
-//   warps 2-9  epilogue: tcgen05.ld 32 lanes x 32 columns per warp, alpha/beta
-//              and the store to C (rows of TMEM lane quadrant warp%4, columns split
-//              in two halves).
+//   warps 2-9 or 2-17 epilogue: tcgen05.ld 32 lanes x 32 columns per warp, alpha/beta
+//              and the store to C (rows of TMEM lane quadrant warp%4, columns split in
+//              halves or quarters; see epi_warps for which).
 // Every mbarrier wait is bounded by the global timer; on expiry the kernel writes
 // its error word, lets in-flight copies and MMAs finish (bounded), frees its tensor
 // memory and returns.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
@@ -58,9 +59,9 @@ namespace {
 constexpr int BM = 128;  // UMMA M (one TMEM lane per output row)
 constexpr int BK = 64;   // 64 bfloat16 = 128 bytes = one swizzle row
 constexpr int BK8 = 128; // 128 e4m3 = 128 bytes = one swizzle row
-constexpr int kEpiWarps = 8;
-constexpr int kMaxSmemProblems = 512;  // grouped launch: problem starts kept in shared memory
-constexpr int kThreadsTc = 64 + 32 * kEpiWarps;
+constexpr int kMaxEpiWarps = 16;
+constexpr int kMaxSmemProblems = 448;  // grouped launch: problem starts kept in shared memory
+constexpr int threads_tc(int epi_warps) { return 64 + 32 * epi_warps; }
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
 constexpr unsigned long long kDrainLimitNs = 200000000ull;  // 0.2 s
 
@@ -386,11 +387,20 @@ static_assert(prod_coll(6, 0) == 1 && prod_coll(6, 1) == 2 && prod_coll(6, 2) ==
 // C0 and X are read through the non-coherent read-only path: within the kernel every
 // element of C0 is read once, by the thread that later overwrites it when C aliases C0,
 // and X is never written, so these loads need not wait behind earlier stores.
-// Shared-memory staging of the epilogue: one 32 x 16 binary32 block per warp, rows 80
-// bytes apart, so that both the row-per-lane writes and the row-major reads are free of
-// bank conflicts (one two-way conflict on the reads).
-constexpr int kStgStride = 20;                       // floats per staged row
-constexpr uint32_t kStgBytes = 32 * kStgStride * 4;  // per epilogue warp
+// Shared-memory staging of the epilogue: one 32 x 16 binary32 block per warp, laid out so that
+// the row-per-lane writes and the row-major reads are free of bank conflicts: with eight
+// epilogue warps rows 80 bytes apart; with sixteen, whose blocks have to fit next to the ring,
+// 64-byte rows with quad c of row r at quad slot c ^ (r / 2 % 4).
+template <int EW>
+struct Stg {
+    static constexpr int ROW = EW <= 8 ? 20 : 16;               // floats from row to row
+    static constexpr uint32_t BYTES = 32 * ROW * 4;             // per epilogue warp
+    // quad c of row r; column j of row r
+    static __device__ __forceinline__ int quad(int r, int c) {
+        return EW <= 8 ? r * ROW + 4 * c : r * ROW + ((c ^ ((r >> 1) & 3)) << 2);
+    }
+    static __device__ __forceinline__ int at(int r, int j) { return EW <= 8 ? r * ROW + j : quad(r, j >> 2) + (j & 3); }
+};
 
 // Final values of 32 columns [gcol, gcol + 32) of the warp's 32 rows (row0 + lane holds
 // v[0..31], a row per lane as tensor memory delivers them): alpha v + beta C0 stored to C,
@@ -399,7 +409,9 @@ constexpr uint32_t kStgBytes = 32 * kStgStride * 4;  // per epilogue warp
 // consecutive columns per lane in 16-byte accesses where rows are 16-byte aligned, one
 // column per lane (16 lanes per row) elsewhere -- so that C0, X, C and D move in 64-byte
 // row segments; every element is formed with the same operations as in the separate loops.
-template <bool MAYFUSE = true>  // false: the chain code is left out (FP8 never carries one)
+// MAYFUSE false: the chain code is left out (FP8 never carries one); ANYROW false: rows are known to
+// be 16-byte aligned.
+template <int EW, bool MAYFUSE, bool ANYROW>
 __device__ __forceinline__ void store_staged32(const EpiArgs& e, int64_t row0, int64_t gcol, const float* v,
                                                float* stg, int lane, double* sq) {
     const bool fuse = MAYFUSE && e.fuse != 0;
@@ -409,10 +421,10 @@ __device__ __forceinline__ void store_staged32(const EpiArgs& e, int64_t row0, i
         __syncwarp();  // the previous half's reads are done
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            *reinterpret_cast<float4*>(stg + lane * kStgStride + 4 * j) =
+            *reinterpret_cast<float4*>(stg + Stg<EW>::quad(lane, j)) =
                 make_float4(v[16 * h + 4 * j], v[16 * h + 4 * j + 1], v[16 * h + 4 * j + 2], v[16 * h + 4 * j + 3]);
         __syncwarp();
-        if (e.vec) {
+        if (!ANYROW || e.vec) {
             // rows of a multiple of four floats, 16-byte aligned: lane (row group lane / 4,
             // quadruple lane % 4) moves four consecutive columns of rows lane / 4 + 8 it in
             // 16-byte accesses (a quadruple is wholly inside or outside the N columns)
@@ -440,7 +452,7 @@ __device__ __forceinline__ void store_staged32(const EpiArgs& e, int64_t row0, i
 #pragma unroll
                 for (int q = 0; q < 4; ++q) dd[it][q] = 0.0f;
                 if (!cin || grow >= e.M) continue;
-                const float4 a = *reinterpret_cast<const float4*>(stg + r * kStgStride + 4 * cq);
+                const float4 a = *reinterpret_cast<const float4*>(stg + Stg<EW>::quad(r, cq));
                 const float av[4] = {a.x, a.y, a.z, a.w};
                 const float c0v[4] = {c0p[it].x, c0p[it].y, c0p[it].z, c0p[it].w};
                 const float xv[4] = {xp[it].x, xp[it].y, xp[it].z, xp[it].w};
@@ -468,51 +480,74 @@ __device__ __forceinline__ void store_staged32(const EpiArgs& e, int64_t row0, i
 #pragma unroll
                 for (int it = 0; it < 4; ++it) {
                     const int r = it * 8 + (lane >> 2);
-                    *reinterpret_cast<float4*>(stg + r * kStgStride + 4 * cq) =
+                    *reinterpret_cast<float4*>(stg + Stg<EW>::quad(r, cq)) =
                         make_float4(dd[it][0], dd[it][1], dd[it][2], dd[it][3]);
                 }
             }
-        } else {
+        } else if constexpr (ANYROW) {
             // rows of any length: lane (j = lane % 16, rh = lane / 16) takes column j of this
             // half in rows rh, rh + 2, ..., rh + 30, so that every access of the warp covers two
-            // 64-byte row segments whatever the rows' alignment; the loads of eight rows go out
+            // 64-byte row segments whatever the rows' alignment; all of the half's loads go out
             // before any is used; D goes back into the element's own staging slot (its lane
             // owns it)
             const int j = lane & 15, rh = lane >> 4;
             const int64_t col = gcol + 16 * h + j;
             const bool cin = col < e.N;
-#pragma unroll 1
-            for (int b8 = 0; b8 < 2; ++b8) {
-                float t[8], u[8];
+            if constexpr (!MAYFUSE) {
+                // no chain: all sixteen rows' C0 in flight
+                const int64_t step = 2 * (e.ldc > 0 ? e.ldc : (int64_t)e.N);  // two rows on
+                const int rows_in = e.M - row0 < 32 ? (int)(e.M - row0) : 32;  // rows of the block inside M
+                int64_t off = (row0 + rh) * (step / 2) + col;
+                float t[16];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int64_t grow = row0 + rh + 2 * (8 * b8 + k);
+                for (int k = 0; k < 16; ++k, off += step) {
                     t[k] = 0.0f;
-                    u[k] = 0.0f;
-                    if (cin && grow < e.M) {
-                        const int64_t base = grow * (e.ldc > 0 ? e.ldc : (int64_t)e.N) + col;
-                        if (e.beta != 0.0f) t[k] = __ldg(e.C0 + base);
-                        if (fuse) u[k] = __ldg(e.X + base);
+                    if (cin && rh + 2 * k < rows_in && e.beta != 0.0f) t[k] = __ldg(e.C0 + off);
+                }
+                off -= 16 * step;
+                asm volatile("" : "+l"(off));  // the offsets are formed again, not kept: sixteen of them would spill
+#pragma unroll
+                for (int k = 0; k < 16; ++k, off += step) {
+                    if (cin && rh + 2 * k < rows_in) {
+                        float o = e.alpha * stg[Stg<EW>::at(rh + 2 * k, j)];
+                        if (e.beta != 0.0f) o = fmaf(e.beta, t[k], o);
+                        e.C[off] = o;
                     }
                 }
+            } else {
+#pragma unroll 1
+                for (int b8 = 0; b8 < 2; ++b8) {
+                    float t[8], u[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int r = rh + 2 * (8 * b8 + k);
-                    const int64_t grow = row0 + r;
-                    float dv = 0.0f;
-                    if (cin && grow < e.M) {
-                        const int64_t base = grow * (e.ldc > 0 ? e.ldc : (int64_t)e.N) + col;
-                        float o = e.alpha * stg[r * kStgStride + j];
-                        if (e.beta != 0.0f) o = fmaf(e.beta, t[k], o);
-                        e.C[base] = o;
-                        if (fuse) {
-                            dv = fmaf(e.alpha2, u[k], o);  // D = C + alpha2 X, one rounding
-                            e.D[base] = dv;
-                            if (k & 1) s3 = fmaf(dv, dv, s3);
-                            else s2 = fmaf(dv, dv, s2);
+                    for (int k = 0; k < 8; ++k) {
+                        const int64_t grow = row0 + rh + 2 * (8 * b8 + k);
+                        t[k] = 0.0f;
+                        u[k] = 0.0f;
+                        if (cin && grow < e.M) {
+                            const int64_t base = grow * (e.ldc > 0 ? e.ldc : (int64_t)e.N) + col;
+                            if (e.beta != 0.0f) t[k] = __ldg(e.C0 + base);
+                            if (fuse) u[k] = __ldg(e.X + base);
                         }
                     }
-                    if (fuse) stg[r * kStgStride + j] = dv;  // rows >= M and columns >= N staged as +0
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int r = rh + 2 * (8 * b8 + k);
+                        const int64_t grow = row0 + r;
+                        float dv = 0.0f;
+                        if (cin && grow < e.M) {
+                            const int64_t base = grow * (e.ldc > 0 ? e.ldc : (int64_t)e.N) + col;
+                            float o = e.alpha * stg[Stg<EW>::at(r, j)];
+                            if (e.beta != 0.0f) o = fmaf(e.beta, t[k], o);
+                            e.C[base] = o;
+                            if (fuse) {
+                                dv = fmaf(e.alpha2, u[k], o);  // D = C + alpha2 X, one rounding
+                                e.D[base] = dv;
+                                if (k & 1) s3 = fmaf(dv, dv, s3);
+                                else s2 = fmaf(dv, dv, s2);
+                            }
+                        }
+                        if (fuse) stg[Stg<EW>::at(r, j)] = dv;  // rows >= M and columns >= N staged as +0
+                    }
                 }
             }
         }
@@ -529,8 +564,11 @@ __device__ __forceinline__ void store_staged32(const EpiArgs& e, int64_t row0, i
                 float x[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float* col = stg + (4 * (4 * hb + k)) * kStgStride + cc;
-                    x[k] = (col[0] + col[kStgStride]) + (col[2 * kStgStride] + col[3 * kStgStride]);
+                    // (sixteen warps: the second half-warp reads each pair of rows the other way
+                    // round, rows of opposite parity, so that no two lanes share a bank)
+                    const int r = 4 * (4 * hb + k), f = EW <= 8 ? 0 : hb;
+                    x[k] = (stg[Stg<EW>::at(r + f, cc)] + stg[Stg<EW>::at(r + 1 - f, cc)]) +
+                           (stg[Stg<EW>::at(r + 2 + f, cc)] + stg[Stg<EW>::at(r + 3 - f, cc)]);
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) x[k] += __shfl_xor_sync(0xffffffffu, x[k], 16);  // q_k + q_k+4
@@ -542,7 +580,7 @@ __device__ __forceinline__ void store_staged32(const EpiArgs& e, int64_t row0, i
             if (grow < e.M) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float4 d = *reinterpret_cast<const float4*>(stg + lane * kStgStride + 4 * j);
+                    const float4 d = *reinterpret_cast<const float4*>(stg + Stg<EW>::quad(lane, j));
                     const float dv[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -560,7 +598,7 @@ __device__ __forceinline__ void store_staged32(const EpiArgs& e, int64_t row0, i
 // PAIR: a cluster of two CTAs computes a 256 x BN tile with M = 256 MMAs issued by the first
 // CTA; each CTA holds 128 rows of A and BN / 2 rows of B^T per stage (the pair's B tile is
 // split by columns), and 128 rows of the accumulator in its own tensor memory.
-template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false, bool PAIR = false>
+template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, bool PAIR, int EW>
 struct TcCfg {
     static constexpr uint32_t A_TILE = BM * 128;  // 128 rows x 128 bytes
     static constexpr uint32_t B_TILE = (PAIR ? BN / 2 : BN) * 128;
@@ -582,14 +620,16 @@ struct TcCfg {
     static constexpr uint32_t TMEM_COLS = COLS <= 32 ? 32 : COLS <= 64 ? 64 : COLS <= 128 ? 128 : COLS <= 256 ? 256
                                                                                                               : 512;
     static constexpr uint32_t NBARS = 2 * STAGES + 2 * ACC + 1;
-    static constexpr int EPI_ARRIVALS = (PAIR ? 2 : 1) * kEpiWarps;  // per drained accumulator
-    static constexpr uint32_t STG = kEpiWarps * kStgBytes;  // epilogue staging blocks
+    static constexpr int EPI_COLS = BN / (EW / 4);                   // columns of an epilogue warp
+    static constexpr int THREADS = threads_tc(EW);
+    static constexpr int EPI_ARRIVALS = (PAIR ? 2 : 1) * EW;         // per drained accumulator
+    static constexpr uint32_t STG = EW * Stg<EW>::BYTES;  // epilogue staging blocks
     // FP8: scale-factor blocks of every stage (A's, then BN / 128 of B's), after the tiles
     static constexpr uint32_t SF_STAGE = FP8 ? (uint32_t)kSfBlock * (1 + BN / 128) : 0;
     static constexpr size_t SMEM = 1024 /*align slack*/ + (size_t)STAGES * (STAGE + SF_STAGE) + STG + 8 * NBARS + 16;
     static_assert(SMEM <= 232448, "shared memory per CTA");
     static_assert(COLS <= 512, "accumulators exceed tensor memory");
-    static_assert(BN % 64 == 0 && BN >= 64 && BN <= 256, "BN");
+    static_assert(BN % (8 * EW) == 0 && BN <= 256, "whole 32-column groups per epilogue warp");
     static_assert(!CHUNKED || BN <= 128, "chunked sums live in registers: BN <= 128");
     static_assert(!FP8 || (!CHUNKED && NPROD == 1 && PA == 1 && PB == 1), "FP8 runs one plane, scaled in the MMA");
     static_assert(!CHUNKED || ACC == 2, "K chunks drain the accumulator while the next chunk runs");
@@ -623,6 +663,7 @@ struct TileInfo {
 
 // Tiles of one problem (kernel arguments).
 struct OneProblem {
+    static constexpr bool kGrouped = false;
     const CUtensorMap* ta;
     const CUtensorMap* tb;
     EpiArgs ep;
@@ -652,6 +693,7 @@ struct OneProblem {
 // Tiles of a grouped launch: tile t belongs to the problem whose range holds t
 // (binary search over tile_start, which increases along the table).
 struct ProblemTable {
+    static constexpr bool kGrouped = true;
     const TcProblem* probs;
     int nprob, bn;
     const int* starts;  // shared-memory copy of every problem's tile_start (null: read probs)
@@ -686,9 +728,9 @@ struct ProblemTable {
 // shared-memory stage ring and the two tensor-memory accumulator buffers carry on
 // from tile to tile, so the producer runs ahead into the next tile and the MMAs of a
 // tile overlap the epilogue of the previous one.
-template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, bool PAIR, class Src>
+template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, bool PAIR, int EW, class Src>
 __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_tiles, int* err) {
-    using Cfg = TcCfg<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, PAIR>;
+    using Cfg = TcCfg<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, PAIR, EW>;
     constexpr uint32_t IDESC = idesc_bf16<BN, Cfg::TILE_M>();
     // a CTA pair serves tile c, c + clusters, ... (c = its cluster); its second CTA (rank 1)
     // holds rows 128..255 of each tile and columns BN / 2.. of each B tile
@@ -913,13 +955,14 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
         __syncwarp();
     } else {
         // ---- epilogue ----
+        constexpr int kEpiCols = Cfg::EPI_COLS;
         const int ew = warp - 2;
         const int q = warp & 3;  // TMEM lane quadrant this warp may access
-        const int half = ew >> 2;
-        const int colbase = half * (BN / 2);
+        const int colbase = (ew >> 2) * kEpiCols;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
-        float* stg = stg_all + ew * (kStgBytes / 4);
-        constexpr int G = BN / 2 / 32;  // 32-column groups per thread
+        float* stg = stg_all + ew * (Stg<EW>::BYTES / 4);
+        constexpr int G = kEpiCols / 32;  // 32-column groups per thread
+        constexpr bool ANYROW = EW > 8 || Src::kGrouped;  // eight warps in a launch of its own: see epi_warps
         int gc = 0;
         bool ok = true;
         for (int t = first_tile; t < total_tiles && ok; t += tile_step) {
@@ -934,9 +977,9 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
             // K chunks sum in registers; a single accumulator buffer is copied to registers
             // and released before the stores, so that the next tile's MMAs start at once
             constexpr bool HOLD = CHUNKED || ACC == 1;
-            float sum[HOLD ? BN / 2 : 1];
+            float sum[HOLD ? kEpiCols : 1];
 #pragma unroll
-            for (int i = 0; i < (HOLD ? BN / 2 : 1); ++i) sum[i] = 0.0f;
+            for (int i = 0; i < (HOLD ? kEpiCols : 1); ++i) sum[i] = 0.0f;
             for (int c = 0; c < nchunks; ++c, ++gc) {
                 const int ab = ACC == 1 ? 0 : gc & 1;
                 const uint32_t aph = (uint32_t)(ACC == 1 ? gc : gc >> 1) & 1u;
@@ -945,7 +988,7 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
                     // bringing it into L2 a chunk or two ahead
                     const int64_t off = grow * (ep.ldc > 0 ? ep.ldc : (int64_t)ep.N) + n0 + colbase;
 #pragma unroll
-                    for (int k = 0; k < BN / 2; k += 32) {
+                    for (int k = 0; k < kEpiCols; k += 32) {
                         if (ep.beta != 0.0f) prefetch_l2(ep.C0 + off + k);
                         if (ep.fuse) prefetch_l2(ep.X + off + k);
                     }
@@ -978,7 +1021,7 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
 #pragma unroll
                         for (int i = 0; i < 32; ++i) sum[g * 32 + i] = v[i];
                     } else {
-                        store_staged32<!FP8>(ep, row0, (int64_t)n0 + colbase + g * 32, v, stg, lane, &sq);
+                        store_staged32<EW, !FP8, ANYROW>(ep, row0, (int64_t)n0 + colbase + g * 32, v, stg, lane, &sq);
                     }
                 }
                 tc_fence_before();
@@ -992,7 +1035,7 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
                 if (ok) {
 #pragma unroll
                     for (int g = 0; g < G; ++g)
-                        store_staged32<!FP8>(ep, row0, (int64_t)n0 + colbase + g * 32, sum + g * 32, stg, lane, &sq);
+                        store_staged32<EW, !FP8, ANYROW>(ep, row0, (int64_t)n0 + colbase + g * 32, sum + g * 32, stg, lane, &sq);
                 }
             }
             if (ep.fuse && ok) {  // fixed butterfly over the warp's rows, one partial per warp
@@ -1001,7 +1044,7 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
                 // one slot per (128-row tile, column tile, warp) in row-major tile order, so that
                 // CTA pairs and single CTAs sum the same partials in the same order
                 const int64_t tile128 = (int64_t)((ti.m0 + (int)rank * BM) / BM) * ti.tiles_n + ti.n0 / BN;
-                if (lane == 0 && ep.frob_part) ep.frob_part[tile128 * kEpiWarps + ew] = sq;
+                if (lane == 0 && ep.frob_part) ep.frob_part[tile128 * EW + ew] = sq;
             }
             if (ti.span_end && ok && lane == 0) {
                 __threadfence();  // the warp's stores of this tile come first
@@ -1021,30 +1064,30 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
     }
 }
 
-template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8>
-__global__ void __launch_bounds__(kThreadsTc, 1)
+template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, int EW>
+__global__ void __launch_bounds__(threads_tc(EW), 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiArgs ep,
                    int Mp, int Np, int num_kb, int chunk_kb, int tiles_m, int tiles_n, int group, int pf_kb,
                    int* err) {
     const OneProblem src{&tmA, &tmB, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group, BN, pf_kb, BM};
-    gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, false>(src, tiles_m * tiles_n, err);
+    gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, false, EW>(src, tiles_m * tiles_n, err);
 }
 
 // The same GEMM on CTA pairs: tiles of 256 x BN rows (tiles_m counts 256-row tiles).
 // FP8: tmSA / tmSB are the scale-factor blocks of A and B (unused otherwise).
-template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsTc, 1)
+template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, int EW>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_tc(EW), 1)
     gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmSA, const __grid_constant__ CUtensorMap tmSB, EpiArgs ep,
                         int Mp, int Np, int num_kb, int chunk_kb, int tiles_m, int tiles_n, int group, int pf_kb,
                         int* err) {
     const OneProblem src{&tmA,  &tmB, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group, BN, pf_kb, 2 * BM,
                          &tmSA, &tmSB};
-    gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, true>(src, tiles_m * tiles_n, err);
+    gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, true, EW>(src, tiles_m * tiles_n, err);
 }
 
-template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8>
-__global__ void __launch_bounds__(kThreadsTc, 1)
+template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, int EW>
+__global__ void __launch_bounds__(threads_tc(EW), 1)
     gemm_tc_grouped_kernel(const TcProblem* __restrict__ probs, int nprob, int total_tiles, int* err) {
     // every role looks up its tile's problem by binary search over the problems' first
     // tiles: keep them in shared memory (the persistent body synchronises the block
@@ -1054,7 +1097,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
     if (in_smem)
         for (int i = threadIdx.x; i < nprob; i += blockDim.x) s_starts[i] = probs[i].tile_start;
     const ProblemTable src{probs, nprob, BN, in_smem ? s_starts : nullptr};
-    gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, false>(src, total_tiles, err);
+    gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, false, EW>(src, total_tiles, err);
 }
 
 // Frobenius norm of a fused chain: the per-warp partials summed in index order by one
@@ -1477,12 +1520,12 @@ bool make_map(CUtensorMap* map, void* base, int64_t inner, int64_t rows, int box
     return true;
 }
 
-template <int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false>
+template <int EW, int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false>
 cudaError_t launch_mma(const CUtensorMap& ta, const CUtensorMap& tb, const EpiArgs& ep, int Mp, int Np, int num_kb,
                        int chunk_kb, int group, int pf_kb, int* err, cudaStream_t st) {
     // Np is the plane stride (a multiple of 256); only ceil(N / BN) column tiles hold data
-    using Cfg = TcCfg<BN, P, P, NPROD, STAGES, CHUNKED, FP8>;
-    auto kern = gemm_tc_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8>;
+    using Cfg = TcCfg<BN, P, P, NPROD, STAGES, CHUNKED, FP8, false, EW>;
+    auto kern = gemm_tc_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8, EW>;
     static bool attr_set = false;  // per instantiation
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
@@ -1493,19 +1536,19 @@ cudaError_t launch_mma(const CUtensorMap& ta, const CUtensorMap& tb, const EpiAr
     const int64_t total = (int64_t)tiles_m * tiles_n;
     if (total > 0x7fffffff) return cudaErrorInvalidValue;
     const int64_t grid = std::min<int64_t>(total, (int64_t)sm_count());  // persistent: one CTA per SM
-    kern<<<(unsigned)grid, kThreadsTc, Cfg::SMEM, st>>>(ta, tb, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group,
+    kern<<<(unsigned)grid, Cfg::THREADS, Cfg::SMEM, st>>>(ta, tb, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group,
                                                         pf_kb, err);
     return cudaGetLastError();
 }
 
 
 // The pair kernel: Mp a multiple of 256; one cluster of two CTAs per two SMs.
-template <int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false>
+template <int EW, int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false>
 cudaError_t launch_mma_pair(const CUtensorMap& ta, const CUtensorMap& tb, const EpiArgs& ep, int Mp, int Np,
                             int num_kb, int chunk_kb, int group, int pf_kb, int* err, cudaStream_t st,
                             const CUtensorMap* tsa = nullptr, const CUtensorMap* tsb = nullptr) {
-    using Cfg = TcCfg<BN, P, P, NPROD, STAGES, CHUNKED, FP8, true>;
-    auto kern = gemm_tc_pair_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8>;
+    using Cfg = TcCfg<BN, P, P, NPROD, STAGES, CHUNKED, FP8, true, EW>;
+    auto kern = gemm_tc_pair_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8, EW>;
     if (FP8 && !(tsa && tsb)) return cudaErrorInvalidValue;
     static bool attr_set = false;  // per instantiation
     if (!attr_set) {
@@ -1523,7 +1566,7 @@ cudaError_t launch_mma_pair(const CUtensorMap& ta, const CUtensorMap& tb, const 
     if (max_clusters == 0) {
         cudaLaunchConfig_t lc = {};
         lc.gridDim = dim3((unsigned)(sm_count() & ~1));
-        lc.blockDim = dim3(kThreadsTc);
+        lc.blockDim = dim3(Cfg::THREADS);
         lc.dynamicSmemBytes = Cfg::SMEM;
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, kern, &lc) != cudaSuccess || n <= 0) {
@@ -1533,7 +1576,7 @@ cudaError_t launch_mma_pair(const CUtensorMap& ta, const CUtensorMap& tb, const 
         max_clusters = std::min(n, sm_count() / 2);
     }
     const int64_t clusters = std::min<int64_t>(total, (int64_t)max_clusters);
-    kern<<<(unsigned)(2 * clusters), kThreadsTc, Cfg::SMEM, st>>>(ta, tb, FP8 ? *tsa : ta, FP8 ? *tsb : tb, ep, Mp,
+    kern<<<(unsigned)(2 * clusters), Cfg::THREADS, Cfg::SMEM, st>>>(ta, tb, FP8 ? *tsa : ta, FP8 ? *tsb : tb, ep, Mp,
                                                                   Np, num_kb, chunk_kb, tiles_m, tiles_n, group,
                                                                   pf_kb, err);
     return cudaGetLastError();
@@ -1542,6 +1585,18 @@ cudaError_t launch_mma_pair(const CUtensorMap& ta, const CUtensorMap& tb, const 
 cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N, int64_t K,
                             float alpha, float beta, int tile_cfg, void* scratch, size_t scratch_bytes, int* err,
                             cudaStream_t st, TcEvents& ev, std::string* why);
+
+// Epilogue warps of a launch.  An epilogue bound by the latency of its C0 / X loads and staging
+// round trips takes sixteen: rows that are not 16-byte aligned, a word a lane (GEMM with
+// 8 -> 16 warps, us: 4001 x 500 x 3003, two terms 82 -> 60; FP8 3000 x 4100 x 5003 100 -> 88; six-loop chain at
+// 4095, three terms 611 -> 573), and the chain behind a single product, whose MMAs are too few
+// to hide it (4096^3 185 -> 162).  Elsewhere eight: the MMAs hide the rest, and sixteen warps'
+// 112 registers a thread cost 1 to 2% (4096^3 aligned, two or three terms, chain or not).
+int epi_warps(bool vec, bool fuse, int planes) { return !vec || (fuse && planes == 1) ? 16 : 8; }
+// ... of a grouped launch, whose problems' rows are of any alignment: sixteen where some problem
+// carries a chain and the products are few (the 16-program suite, three products: 180 us against
+// 196; six products: 283 against 265; without chains 148 against 134).
+int grouped_epi_warps(int prec, bool chain) { return chain && prec != GAO_GEMM_BF16X6 && prec != GAO_GEMM_FP8 ? 16 : 8; }
 
 }  // namespace
 
@@ -1567,7 +1622,7 @@ Fp8Layout fp8_layout(int64_t M, int64_t N, int64_t K) {
 }
 
 // Planes (or FP8 arrays) first, then binary64 partials for a fused chain's norm
-// (8 per 128 x 128 tile), then its row sums' 32-row block values (binary32, [Mp / 32][N]).
+// (16 per 128 x 128 tile), then its row sums' 32-row block values (binary32, [Mp / 32][N]).
 size_t tc_planes_bytes(int prec, int64_t M, int64_t N, int64_t K) {
     if (prec == GAO_GEMM_FP8) return fp8_layout(M, N, K).total;
     if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_BF16X6) return 0;
@@ -1580,7 +1635,7 @@ size_t tc_planes_bytes(int prec, int64_t M, int64_t N, int64_t K) {
 
 size_t tc_frob_partials_bytes(int64_t M, int64_t N) {
     const int64_t tiles = (ru(std::max<int64_t>(M, 1), 2 * BM) / BM) * ((std::max<int64_t>(N, 1) + 127) / 128);
-    return (size_t)ru(tiles * kEpiWarps * (int64_t)sizeof(double), 1024);
+    return (size_t)ru(tiles * kMaxEpiWarps * (int64_t)sizeof(double), 1024);
 }
 
 size_t tc_partials_bytes(int64_t M, int64_t N) {
@@ -1763,13 +1818,14 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
     float* rpart = reinterpret_cast<float*>(reinterpret_cast<char*>(fpart) + tc_frob_partials_bytes(Mlay, N));
     const int64_t tiles_n = (N + bn - 1) / bn;
     ep.ldE = M;
+    const int ew = epi_warps(ep.vec != 0, fuse != nullptr, P);
     if (fuse) {
         ep.X = fuse->X;
         ep.D = fuse->D;
         ep.E = fuse->E;
         ep.ldE = fuse->ldE > 0 ? fuse->ldE : M;
         ep.alpha2 = fuse->alpha2;
-        ep.frob_part = fuse->frob_out ? fpart + (part ? part->row_tile0 : 0) * tiles_n * kEpiWarps : nullptr;
+        ep.frob_part = fuse->frob_out ? fpart + (part ? part->row_tile0 : 0) * tiles_n * ew : nullptr;
         ep.rsum_part = fuse->rowsum_out ? rpart + (part ? part->row_tile0 : 0) * (BM / kRowsumBlock) * N : nullptr;
         ep.ldR = N;
         ep.fuse = 1;
@@ -1777,40 +1833,32 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
     if (ev.k0) record_timing(ev.k0, st);
     cudaError_t e;
     const int mp = (int)Mp, np = (int)Np;
-    if (pair) {
-        // stages per variant: as many as fit next to the epilogue's staging blocks
-        if (P == 3)
-            e = chunked ? launch_mma_pair<128, 3, 6, 2, true>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st)
-                        : launch_mma_pair<128, 3, 6, 2, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err,
-                                                               st);
-        else if (P == 2)
-            e = chunked ? launch_mma_pair<128, 2, 3, 4, true>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st)
-                        : launch_mma_pair<128, 2, 3, 4, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err,
-                                                               st);
-        else if (chunked)
-            e = launch_mma_pair<128, 1, 1, 8, true>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
-        else if (bn == 256)
-            e = launch_mma_pair<256, 1, 1, 6, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
-        else
-            e = launch_mma_pair<128, 1, 1, 8, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
-    } else if (P == 3)
-        e = chunked ? launch_mma<128, 3, 6, 2, true>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st)
-                    : launch_mma<128, 3, 6, 2, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
-    else if (P == 2)
-        e = chunked ? launch_mma<128, 2, 3, 3, true>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st)
-                    : launch_mma<128, 2, 3, 3, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
-    else if (chunked)
-        e = launch_mma<128, 1, 1, 6, true>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
-    else if (bn == 256)
-        e = launch_mma<256, 1, 1, 4, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
-    else
-        e = launch_mma<128, 1, 1, 6, false>(ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st);
+    // stages per variant: as many as fit next to the epilogue's staging blocks
+#define GAO_TC_ARGS ta, tb, ep, mp, np, num_kb, chunk_kb, group, pf_kb, err, st
+#define GAO_TC_LAUNCH(EW)                                                                                            \
+    (pair ? (P == 3   ? (chunked ? launch_mma_pair<EW, 128, 3, 6, 2, true>(GAO_TC_ARGS)                               \
+                                 : launch_mma_pair<EW, 128, 3, 6, 2, false>(GAO_TC_ARGS))                             \
+             : P == 2 ? (chunked ? launch_mma_pair<EW, 128, 2, 3, 4, true>(GAO_TC_ARGS)                               \
+                                 : launch_mma_pair<EW, 128, 2, 3, 4, false>(GAO_TC_ARGS))                             \
+             : chunked   ? launch_mma_pair<EW, 128, 1, 1, 8, true>(GAO_TC_ARGS)                                       \
+             : bn == 256 ? launch_mma_pair<EW, 256, 1, 1, 6, false>(GAO_TC_ARGS)                                      \
+                         : launch_mma_pair<EW, 128, 1, 1, 8, false>(GAO_TC_ARGS))                                     \
+          : (P == 3   ? (chunked ? launch_mma<EW, 128, 3, 6, 2, true>(GAO_TC_ARGS)                                    \
+                                 : launch_mma<EW, 128, 3, 6, 2, false>(GAO_TC_ARGS))                                  \
+             : P == 2 ? (chunked ? launch_mma<EW, 128, 2, 3, 3, true>(GAO_TC_ARGS)                                    \
+                                 : launch_mma<EW, 128, 2, 3, 3, false>(GAO_TC_ARGS))                                  \
+             : chunked   ? launch_mma<EW, 128, 1, 1, 6, true>(GAO_TC_ARGS)                                            \
+             : bn == 256 ? launch_mma<EW, 256, 1, 1, 4, false>(GAO_TC_ARGS)                                           \
+                         : launch_mma<EW, 128, 1, 1, 6, false>(GAO_TC_ARGS)))
+    e = ew == 16 ? GAO_TC_LAUNCH(16) : GAO_TC_LAUNCH(8);
+#undef GAO_TC_LAUNCH
+#undef GAO_TC_ARGS
     if (e != cudaSuccess) return e;
     ev.launches += 1;
     if (ev.k1) record_timing(ev.k1, st);
     if (fuse && fuse->frob_out && (!part || part->last)) {
         const int64_t tiles = (ru(Mlay, BM) / BM) * tiles_n;  // every block's tiles
-        frob_partials_kernel<<<1, 256, 0, st>>>(fpart, tiles * kEpiWarps, fuse->frob_out);
+        frob_partials_kernel<<<1, 256, 0, st>>>(fpart, tiles * ew, fuse->frob_out);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         ev.launches += 1;
     }
@@ -1866,20 +1914,32 @@ cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const floa
                reinterpret_cast<const float*>(sa), reinterpret_cast<const float*>(sb), (int)L.kbs, (int)L.Np};
     if (ev.k0) record_timing(ev.k0, st);
     const int kbs = (int)L.kbs;
+    const int ew = epi_warps(ep.vec != 0, false, 1);
     cudaError_t e;
     if (pair) {
         CUtensorMap tsa, tsb;
         if (!make_sf_map(&tsa, sa, L.kbs, L.Mp / 128, 1, why)) return cudaErrorInvalidValue;
         if (!make_sf_map(&tsb, sb, L.kbs, L.Np / 128, bn / 128, why)) return cudaErrorInvalidValue;
-        e = bn == 256 ? launch_mma_pair<256, 1, 1, 6, false, true>(ta, tb, ep, (int)L.Mp, (int)L.Np, kbs, kbs, group, 0,
-                                                                   err, st, &tsa, &tsb)
-                      : launch_mma_pair<128, 1, 1, 8, false, true>(ta, tb, ep, (int)L.Mp, (int)L.Np, kbs, kbs, group, 0,
-                                                                   err, st, &tsa, &tsb);
+        // sixteen epilogue warps' staging leaves room for fewer stages
+        const int mp = (int)L.Mp, np = (int)L.Np;
+        if (ew == 16)
+            e = bn == 256 ? launch_mma_pair<16, 256, 1, 1, 5, false, true>(ta, tb, ep, mp, np, kbs, kbs, group, 0, err, st,
+                                                                           &tsa, &tsb)
+                          : launch_mma_pair<16, 128, 1, 1, 7, false, true>(ta, tb, ep, mp, np, kbs, kbs, group, 0, err, st,
+                                                                           &tsa, &tsb);
+        else
+            e = bn == 256 ? launch_mma_pair<8, 256, 1, 1, 6, false, true>(ta, tb, ep, mp, np, kbs, kbs, group, 0, err, st,
+                                                                          &tsa, &tsb)
+                          : launch_mma_pair<8, 128, 1, 1, 8, false, true>(ta, tb, ep, mp, np, kbs, kbs, group, 0, err, st,
+                                                                          &tsa, &tsb);
     } else {
-        e = bn == 256 ? launch_mma<256, 1, 1, 4, false, true>(ta, tb, ep, (int)L.Mt, (int)L.Np, kbs, kbs, group, 0, err,
-                                                              st)
-                      : launch_mma<128, 1, 1, 6, false, true>(ta, tb, ep, (int)L.Mt, (int)L.Np, kbs, kbs, group, 0, err,
-                                                              st);
+        const int mt = (int)L.Mt, np = (int)L.Np;
+        if (ew == 16)
+            e = bn == 256 ? launch_mma<16, 256, 1, 1, 3, false, true>(ta, tb, ep, mt, np, kbs, kbs, group, 0, err, st)
+                          : launch_mma<16, 128, 1, 1, 5, false, true>(ta, tb, ep, mt, np, kbs, kbs, group, 0, err, st);
+        else
+            e = bn == 256 ? launch_mma<8, 256, 1, 1, 4, false, true>(ta, tb, ep, mt, np, kbs, kbs, group, 0, err, st)
+                          : launch_mma<8, 128, 1, 1, 6, false, true>(ta, tb, ep, mt, np, kbs, kbs, group, 0, err, st);
     }
     if (e != cudaSuccess) return e;
     ev.launches += 1;
@@ -1893,10 +1953,10 @@ cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const floa
 
 namespace {
 
-template <int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false>
+template <int EW, int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false>
 cudaError_t launch_grouped_t(const TcProblem* d_probs, int nprob, int total_tiles, int* err, cudaStream_t st) {
-    using Cfg = TcCfg<BN, P, P, NPROD, STAGES, CHUNKED, FP8>;
-    auto kern = gemm_tc_grouped_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8>;
+    using Cfg = TcCfg<BN, P, P, NPROD, STAGES, CHUNKED, FP8, false, EW>;
+    auto kern = gemm_tc_grouped_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8, EW>;
     static bool attr_set = false;  // per instantiation
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
@@ -1905,7 +1965,7 @@ cudaError_t launch_grouped_t(const TcProblem* d_probs, int nprob, int total_tile
     }
     if (total_tiles <= 0) return cudaSuccess;
     const int grid = std::min(total_tiles, sm_count());  // persistent: one CTA per SM
-    kern<<<(unsigned)grid, kThreadsTc, Cfg::SMEM, st>>>(d_probs, nprob, total_tiles, err);
+    kern<<<(unsigned)grid, Cfg::THREADS, Cfg::SMEM, st>>>(d_probs, nprob, total_tiles, err);
     return cudaGetLastError();
 }
 
@@ -2017,7 +2077,7 @@ cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* s
     float* rpart = reinterpret_cast<float*>(reinterpret_cast<char*>(fpart) + tc_frob_partials_bytes(M, N));
     if (fuse.frob_out) {
         const int64_t tiles = (ru(M, BM) / BM) * ((N + 127) / 128);  // 128 x 128 tiles of the grouped launch
-        frob_partials_kernel<<<1, 256, 0, st>>>(fpart, tiles * kEpiWarps, fuse.frob_out);
+        frob_partials_kernel<<<1, 256, 0, st>>>(fpart, tiles * grouped_epi_warps(prec, true), fuse.frob_out);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         *launches += 1;
@@ -2032,21 +2092,28 @@ cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* s
     return cudaSuccess;
 }
 
-cudaError_t tc_launch_grouped(int prec, bool chunked, const TcProblem* d_probs, int nprob, int total_tiles, int* err,
-                              cudaStream_t st) {
+cudaError_t tc_launch_grouped(int prec, bool chunked, bool chain, const TcProblem* d_probs, int nprob, int total_tiles,
+                              int* err, cudaStream_t st) {
     // nprob == 0 / total_tiles == 0: only sets the kernel's shared-memory attribute
+    const bool wide = grouped_epi_warps(prec, chain) == 16;
     switch (prec) {
         case GAO_GEMM_BF16X6:
-            return chunked ? launch_grouped_t<128, 3, 6, 2, true>(d_probs, nprob, total_tiles, err, st)
-                           : launch_grouped_t<128, 3, 6, 2, false>(d_probs, nprob, total_tiles, err, st);
+            return chunked ? launch_grouped_t<8, 128, 3, 6, 2, true>(d_probs, nprob, total_tiles, err, st)
+                           : launch_grouped_t<8, 128, 3, 6, 2, false>(d_probs, nprob, total_tiles, err, st);
         case GAO_GEMM_BF16X3:
-            return chunked ? launch_grouped_t<128, 2, 3, 3, true>(d_probs, nprob, total_tiles, err, st)
-                           : launch_grouped_t<128, 2, 3, 3, false>(d_probs, nprob, total_tiles, err, st);
+            if (wide)
+                return chunked ? launch_grouped_t<16, 128, 2, 3, 3, true>(d_probs, nprob, total_tiles, err, st)
+                               : launch_grouped_t<16, 128, 2, 3, 3, false>(d_probs, nprob, total_tiles, err, st);
+            return chunked ? launch_grouped_t<8, 128, 2, 3, 3, true>(d_probs, nprob, total_tiles, err, st)
+                           : launch_grouped_t<8, 128, 2, 3, 3, false>(d_probs, nprob, total_tiles, err, st);
         case GAO_GEMM_BF16:
-            return chunked ? launch_grouped_t<128, 1, 1, 6, true>(d_probs, nprob, total_tiles, err, st)
-                           : launch_grouped_t<128, 1, 1, 6, false>(d_probs, nprob, total_tiles, err, st);
+            if (wide)
+                return chunked ? launch_grouped_t<16, 128, 1, 1, 6, true>(d_probs, nprob, total_tiles, err, st)
+                               : launch_grouped_t<16, 128, 1, 1, 6, false>(d_probs, nprob, total_tiles, err, st);
+            return chunked ? launch_grouped_t<8, 128, 1, 1, 6, true>(d_probs, nprob, total_tiles, err, st)
+                           : launch_grouped_t<8, 128, 1, 1, 6, false>(d_probs, nprob, total_tiles, err, st);
         case GAO_GEMM_FP8:
-            return launch_grouped_t<128, 1, 1, 6, false, true>(d_probs, nprob, total_tiles, err, st);
+            return launch_grouped_t<8, 128, 1, 1, 6, false, true>(d_probs, nprob, total_tiles, err, st);
         default:
             return cudaErrorInvalidValue;
     }

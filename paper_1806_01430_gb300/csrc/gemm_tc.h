@@ -19,8 +19,8 @@ struct EpiArgs {
     const float* sb;   // FP8: B's scale-factor blocks [Np / 128][kbs][512 bytes] (read as bytes)
     int kbs, sb_ld;
     // Fused loop chain (fuse != 0): D = C + alpha2 * X written row-major like C, E = D^T
-    // written with row stride M, and per-warp binary64 partials of sum(D^2) (8 per tile,
-    // at frob_part[tile * 8 + epilogue warp]).  D, E, X must not alias C, C0 or each other.
+    // written with row stride M, and per-warp binary64 partials of sum(D^2) (one per epilogue
+    // warp, at frob_part[tile * warps + warp]).  D, E, X must not alias C, C0 or each other.
     const float* X;
     float* D;
     float* E;
@@ -101,8 +101,9 @@ cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* s
 // One launch over nprob problems whose table (tile_start set, in order) is at d_probs
 // in device memory; every problem must come from tc_prepare with the same prec and
 // the same chunked-ness.  total_tiles = sum of tiles_m * tiles_n.  With total_tiles
-// = 0 it only prepares the kernel (shared-memory attribute), launching nothing.
-cudaError_t tc_launch_grouped(int prec, bool chunked, const TcProblem* d_probs, int nprob, int total_tiles, int* err,
-                              cudaStream_t st);
+// = 0 it only prepares the kernel (shared-memory attribute), launching nothing.  chain: some
+// problem of the launch carries a chain (tc_attach_chain); each that does needs it set.
+cudaError_t tc_launch_grouped(int prec, bool chunked, bool chain, const TcProblem* d_probs, int nprob, int total_tiles,
+                              int* err, cudaStream_t st);
 
 }  // namespace gao
