@@ -1100,21 +1100,37 @@ __global__ void __launch_bounds__(threads_tc(EW), 1)
     gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, false, EW>(src, total_tiles, err);
 }
 
-// Frobenius norm of a fused chain: the per-warp partials summed in index order by one
-// block (fixed partition and tree), then the square root.
-__global__ void __launch_bounds__(256) frob_partials_kernel(const double* __restrict__ part, int64_t n,
-                                                            double* __restrict__ out) {
-    __shared__ double w[8];
+// Frobenius norm of a fused chain: the per-warp partials summed by a cluster of eight blocks
+// (fixed partition and tree), then the square root.  One SM completes 1.7 binary64 additions per
+// clock, and a single block took 15 us for the 17672 partials of a 6000 x 6000 result (6.2
+// on eight SMs).
+constexpr int kFrobCtas = 8;
+__global__ void __cluster_dims__(kFrobCtas, 1, 1) __launch_bounds__(128)
+    frob_partials_kernel(const double* __restrict__ part, int64_t n, double* __restrict__ out) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_arrive();  // waited for below: the first block's shared memory is written remotely
+    __shared__ double w[kFrobCtas * 4];
+    constexpr int kAll = kFrobCtas * 128, kAhead = 4;
+    const int t0 = (int)blockIdx.x * 128 + (int)threadIdx.x;
     double t = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) t += part[i];
+    for (int64_t i = t0; i < n; i += kAhead * kAll) {
+        double v[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) v[k] = i + k * kAll < n ? part[i + k * kAll] : 0.0;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) t += v[k];
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double u = 0.0;
-        for (int i = 0; i < 8; ++i) u += w[i];
-        *out = sqrt(u);
+    cluster.barrier_wait();
+    if ((threadIdx.x & 31) == 0) *cluster.map_shared_rank(&w[t0 >> 5], 0) = t;
+    cluster.sync();
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        double u = w[threadIdx.x];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) u += __shfl_xor_sync(0xffffffffu, u, off);
+        if (threadIdx.x == 0) *out = sqrt(u);
     }
 }
 
@@ -1858,7 +1874,7 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
     if (ev.k1) record_timing(ev.k1, st);
     if (fuse && fuse->frob_out && (!part || part->last)) {
         const int64_t tiles = (ru(Mlay, BM) / BM) * tiles_n;  // every block's tiles
-        frob_partials_kernel<<<1, 256, 0, st>>>(fpart, tiles * ew, fuse->frob_out);
+        frob_partials_kernel<<<kFrobCtas, 128, 0, st>>>(fpart, tiles * ew, fuse->frob_out);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         ev.launches += 1;
     }
@@ -2077,7 +2093,7 @@ cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* s
     float* rpart = reinterpret_cast<float*>(reinterpret_cast<char*>(fpart) + tc_frob_partials_bytes(M, N));
     if (fuse.frob_out) {
         const int64_t tiles = (ru(M, BM) / BM) * ((N + 127) / 128);  // 128 x 128 tiles of the grouped launch
-        frob_partials_kernel<<<1, 256, 0, st>>>(fpart, tiles * grouped_epi_warps(prec, true), fuse.frob_out);
+        frob_partials_kernel<<<kFrobCtas, 128, 0, st>>>(fpart, tiles * grouped_epi_warps(prec, true), fuse.frob_out);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         *launches += 1;
