@@ -143,7 +143,8 @@ typedef struct gao_opts {
                                 bits 4-7 log2 of the raster group (0: default 16).  The
                                 default (0) runs plain BF16 without K chunks and FP8 on
                                 256 x 256 pair tiles and the split precisions on 128 x 128
-                                tiles of one CTA; prog_autotune picks one                   */
+                                tiles of one CTA (a large GEMM with its chain: on pairs,
+                                with the prefetch for BF16X6); prog_autotune picks one      */
     int32_t cpu_threads;     /* OpenMP threads for CPU loops (0: all)                       */
     uint64_t seed;           /* seed of the INIT loop's counter hash                        */
     double timeout_s;        /* wall-clock budget of one prog_run (0: none)                 */

@@ -1673,8 +1673,26 @@ struct TcShape {
     int64_t Mp, Np, Kp;
     size_t pb_elems;  // B's planes start this many bfloat16 after A's (room for Mlay rows)
 };
+// The split precisions' default (tile_cfg bits 0-3 zero) for a GEMM with its chain whose result
+// has at least six tiles per SM, over an inner dimension of 1500 or more, with planes of at
+// most 450 MB: CTA pairs, for the three-term split with the L2 prefetch.  The GEMM with its
+// chain, us, one CTA -> this: two terms 6000 x 1500 x 6000 301 -> 283, 6000 x 3000 x 6000
+// 495 -> 471, 4096^3 311 -> 307; three terms 6000 x 2000 x 6000 639 -> 614, 4096^3 565 -> 532,
+// 5000^3 1034 -> 997; 2 to 5% also back to back, at the power cap.  Outside: fewer tiles leave
+// too few 256-row ones to go round (3001 x 1500 x 3003, three terms 162 -> 166); shorter inner
+// dimensions are bound by the epilogue, which a pair's two CTAs run in step (two terms 6000 x
+// 1100 x 6000 240 -> 242, 4001 x 500 x 3003 60 -> 78); larger planes leave nothing to find in L2
+// (8192^3 without a chain, three terms 3761 -> 4091).  Without a chain a pair is up to 6% faster
+// alone, but 1 to 4% slower back to back, where power bounds it.
+bool tc_split_default(int planes, bool chain, int64_t M, int64_t N, int64_t K, int tile_cfg) {
+    return planes > 1 && chain && (tile_cfg & 15) == 0 && K >= 1500 &&
+           ((M + BM - 1) / BM) * ((N + 127) / 128) >= 6 * (int64_t)sm_count() &&
+           (double)planes * (double)(M + N) * (double)K * 2.0 <= 450e6;
+}
+
+// chain: a whole GEMM (no row block) with its chain in the epilogue
 TcShape tc_shape(int prec, int64_t M, int64_t Mlay, int64_t N, int64_t K, int kchunk, int tile_cfg,
-                 const TcPart* part) {
+                 const TcPart* part, bool chain) {
     TcShape g{};
     g.P = planes_of(prec);
     g.Np = ru(N, 256);
@@ -1689,12 +1707,14 @@ TcShape tc_shape(int prec, int64_t M, int64_t Mlay, int64_t N, int64_t K, int kc
     // 2^value row tiles (0: default 16).  The default is the fastest measured shape:
     // 256 x 256 on CTA pairs for the unchunked single product (which the pair's halved B
     // traffic per SM speeds up by 14% at n = 8192), 128 x 128 on one CTA for the split
-    // precisions (a pair gains nothing there).
+    // precisions but for the chains of tc_split_default.
     const int bn_sel = tile_cfg & 3;
     g.bn = 128;
     if (!g.chunked && g.P == 1 && (bn_sel == 2 || bn_sel == 0)) g.bn = 256;
     // a row block must start on a 256-row boundary to run on pairs
-    g.pair = ((tile_cfg & 8) != 0 || (bn_sel == 0 && g.P == 1 && !g.chunked)) && !(part && part->row_tile0 % 2 != 0);
+    g.pair = ((tile_cfg & 8) != 0 || (bn_sel == 0 && g.P == 1 && !g.chunked) ||
+              tc_split_default(g.P, chain, M, N, K, tile_cfg)) &&
+             !(part && part->row_tile0 % 2 != 0);
     g.Mp = ru(M, g.pair ? 2 * BM : BM);
     // A's planes ([P][Mp][Kp], this call's rows) at the start; B's ([P][Np][Kp]) after room
     // for the whole problem's A planes, so that row blocks can share them
@@ -1709,7 +1729,7 @@ cudaError_t tc_init_planes(int prec, int which, int64_t M, int64_t N, int64_t K,
     *launches = 0;
     if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_BF16X6 || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
     if (tc_scratch_bytes(prec, M, N, K) > scratch_bytes || ((uintptr_t)scratch & 1023u)) return cudaErrorInvalidValue;
-    const TcShape g = tc_shape(prec, M, M, N, K, kchunk, tile_cfg, nullptr);
+    const TcShape g = tc_shape(prec, M, M, N, K, kchunk, tile_cfg, nullptr, false);
     __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(scratch);
     if (which == 0) {  // A (M x K) -> [P][Mp][Kp]
         int64_t blocks = (g.Mp * (g.Kp / 8) + 255) / 256;
@@ -1774,12 +1794,13 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
         if (why) *why = "bad column range";
         return cudaErrorInvalidValue;
     }
-    const TcShape g = tc_shape(prec, M, Mlay, N, K, kchunk, tile_cfg, part);
+    const bool chain = fuse && !part;
+    const TcShape g = tc_shape(prec, M, Mlay, N, K, kchunk, tile_cfg, part, chain);
     const int P = g.P, num_kb = g.num_kb, chunk_kb = g.chunk_kb, bn = g.bn;
     const bool chunked = g.chunked, pair = g.pair;
     const int64_t Mp = g.Mp, Np = g.Np, Kp = g.Kp;
     const int group = tc_group_of(tile_cfg);
-    const int pf_kb = tc_prefetch_of(tile_cfg);
+    const int pf_kb = tc_prefetch_of(P == 3 && tc_split_default(P, chain, M, N, K, tile_cfg) ? 4 : tile_cfg);
     if (tc_scratch_bytes(prec, Mlay, N, K) > scratch_bytes || ((uintptr_t)scratch & 1023u)) {
         if (why) *why = "tensor-core scratch too small or misaligned";
         return cudaErrorInvalidValue;

@@ -1,5 +1,6 @@
-"""The epilogue that the tensor-core precisions choose for rows that are not 16-byte aligned
-carries the bits of the same columns in a product with aligned rows."""
+"""The tile shapes and epilogues that the split precisions choose by size, alignment and chain: the
+default carries the bits of the one-CTA tiles (and of the same columns in a product with
+16-byte aligned rows), on both sides of the sizes where it changes."""
 import numpy as np
 import pytest
 
@@ -15,6 +16,35 @@ def gao():
     _build.build()
     import paper_1806_01430_gb300 as g
     return g
+
+
+def chain_program(m, k, n):
+    o = W.OUTPUT
+    bufs = [W.Buffer("A", m, k), W.Buffer("B", k, n), W.Buffer("C", m, n, role=o), W.Buffer("S", m, n),
+            W.Buffer("D", m, n), W.Buffer("E", n, m, role=o), W.Buffer("r", n, 1, role=o),
+            W.Buffer("f", 1, 1, W.F64, o)]
+    L = W.Loop
+    return bufs, [L(W.INIT, [], [0, 1, 2, 3]), L(W.GEMM, [0, 1, 2], [2], 1.5, 0.5), L(W.AXPY, [2, 3], [4], 2.0),
+                  L(W.TRANSPOSE, [4], [5]), L(W.ROWSUM, [5], [6]), L(W.FROBENIUS, [5], [7])]
+
+
+@pytest.mark.parametrize("prec", ["bf16x3", "bf16x6"])
+@pytest.mark.parametrize("m,k,n", [(3968, 1500, 3840), (3968, 1499, 3840), (3841, 1600, 3969), (3840, 1500, 3712),
+                                   (2433, 1500, 3072)])
+def test_chain_default_against_one_cta(gao, prec, m, k, n):
+    bufs, loops = chain_program(m, k, n)
+    got = []
+    for cfg in (0, 1, 9):
+        p = gao.prog_create(bufs, loops, seed=3, gemm_prec=PREC[prec], tile_cfg=cfg, fuse_chains=1)
+        gao.prog_run(p, 0b111111)
+        got.append([gao.prog_output(p, b).copy() for b in (2, 5, 6, 7)])
+        assert gao.prog_stats(p)[1]["launches"] == 5
+        gao.prog_destroy(p)
+    for g in got[1:]:
+        for a, b in zip(got[0][:3], g[:3]):
+            assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
+        # the norm: binary64 partials of the same squares, added in another order
+        assert abs(got[0][3][0, 0] - g[3][0, 0]) <= 1e-12 * abs(g[3][0, 0])
 
 
 @pytest.mark.parametrize("prec", ["bf16", "bf16x3", "bf16x6", "fp8"])
