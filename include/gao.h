@@ -158,7 +158,8 @@ typedef struct gao_opts {
                                 GEMM -> AXPY(C + a X) -> TRANSPOSE [-> ROWSUM] [-> FROBENIUS]
                                 of the transpose (tensor-core BF16 precisions: the GEMM's
                                 epilogue writes C, D, E, the row sums' block values and the
-                                norm's partial sums); linear RELU / SQUARE / AXPY chains;
+                                norm's partial sums); linear RELU / SQUARE / AXPY chains
+                                [-> SUM] [-> COLMAX] of their last value;
                                 STENCIL3 x2 -> SQUARE x2 -> AXPY [-> SUM] [-> COLMAX] of the
                                 magnitude (the gradient chain), with the STENCIL3 that forms
                                 its input joining the pass when it is on the GPU too (one pass
@@ -235,8 +236,9 @@ gao_status prog_run(gao_prog *p, uint64_t gene_mask, uint32_t flags, double *sec
 gao_status prog_output(gao_prog *p, int buf, const void **host_ptr, gao_buffer *shape_out);
 
 /* Device pointer of buffer `buf` (for callers that keep data on the GPU).  A buffer the
- * last run formed only as a GEMM's bfloat16 planes (prog_planes_for) gets its binary32
- * values formed first (the INIT slot alone, on the program's stream, waited for). */
+ * last run formed only as a GEMM's bfloat16 planes (prog_planes_for), or reduced without
+ * writing it (fuse_chains), gets its binary32 values formed first (the INIT slot or the
+ * element-wise chain alone, on the program's stream, waited for). */
 gao_status prog_device_ptr(gao_prog *p, int buf, void **dev_ptr);
 
 /* INIT into GEMM operand planes: a TEMP buffer that an INIT loop writes and that only one

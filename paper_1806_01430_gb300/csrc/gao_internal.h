@@ -149,14 +149,27 @@ struct EwChainOp {
     const float* xa;
     const float* yb;
     float* out;
+    int xi, yi;  // set by the launcher: which of ext[] xa / yb is, -1 for the previous value
 };
 struct EwChain {
     int nops;
-    int vec;  // set by launch_ew_chain
+    int vec;   // set by the launcher
+    int next;  // set by the launcher: distinct arrays the chain reads when there are at most two, else 0
     int64_t n;
+    const float* ext[2];
     EwChainOp op[kMaxChainOps];
 };
 cudaError_t launch_ew_chain(const EwChain& c, cudaStream_t st);
+// A chain over a rows x cols shape (c.n unused) with the sum and / or the column maxima of its
+// last value formed in the same pass (either output may be null; the last op's out null where
+// nothing else reads the value).  Only for shapes ew_chain_reduce_fits accepts.
+struct EwReduce {
+    double* sum_out;
+    float* colmax_out;
+    ReduceScratch scratch;
+};
+bool ew_chain_reduce_fits(int64_t rows, int64_t cols);
+cudaError_t launch_ew_chain_reduce(const EwChain& c, int64_t rows, int64_t cols, const EwReduce& red, cudaStream_t st);
 // Reductions of the gradient chain's m formed in the same pass: the sum (binary64, from one
 // partial per block of the pass in `part`, added in index order) and the column maxima
 // (order-preserving keys in `keys`, one per column, decoded into colmax_out).  Either output

@@ -229,42 +229,127 @@ __global__ void ew_kernel(float* __restrict__ out, const float* __restrict__ x, 
 // The chain is linear: every loop after the first reads the previous loop's value (held
 // in registers) and at most one other buffer from memory; each value is formed with the
 // separate loop's operation, and written only where `out` is set.
-__global__ void ew_chain_kernel(EwChain c) {
+//
+// HBM-bound where its loads are in flight together.  A chain that reads one or two arrays (EXT)
+// loads kAhead quads (kAhead rows' quads in the reducing pass) of each before its first operation,
+// which then picks its operands from registers: fetching an operand when its operation comes
+// makes every operation of the chain wait for memory in turn, and reads an array again each
+// time it is named (the twelve-loop program's four loops on 6000 x 6000 with the last value written: 71.0 -> 64.6 us,
+// 432 MB).
+
+// One operation on N groups of four values: cur = op(x, y), x and y each the previous value or a
+// preloaded array's (EXT), or fetched by `fetch` now.  The branches are uniform: choosing by
+// selects, and forming all three operations, cost ten instructions a value and made the pass
+// issue-bound.
+template <int N>
+__device__ __forceinline__ void chain_axpy(float alpha, float (&cur)[N][4], const float (&x)[N][4], const float (&y)[N][4]) {
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cur[k][q] = ew_apply<Ew::Axpy>(x[k][q], y[k][q], alpha);
+}
+template <bool EXT, int N, class Fetch>
+__device__ __forceinline__ void chain_op(const EwChainOp& op, float (&cur)[N][4], const float (&e0)[N][4],
+                                         const float (&e1)[N][4], const Fetch& fetch) {
+    if (op.kind == 2) {
+        if constexpr (EXT) {
+            if (op.xi < 0) {
+                if (op.yi < 0) chain_axpy(op.alpha, cur, cur, cur);
+                else if (op.yi == 0) chain_axpy(op.alpha, cur, cur, e0);
+                else chain_axpy(op.alpha, cur, cur, e1);
+            } else if (op.xi == 0) {
+                if (op.yi < 0) chain_axpy(op.alpha, cur, e0, cur);
+                else if (op.yi == 0) chain_axpy(op.alpha, cur, e0, e0);
+                else chain_axpy(op.alpha, cur, e0, e1);
+            } else {
+                if (op.yi < 0) chain_axpy(op.alpha, cur, e1, cur);
+                else if (op.yi == 0) chain_axpy(op.alpha, cur, e1, e0);
+                else chain_axpy(op.alpha, cur, e1, e1);
+            }
+        } else {
+            float y[N][4];
+            if (op.yb) {
+                fetch(op.yb, y);
+            } else {
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) y[k][q] = cur[k][q];
+            }
+            if (op.xa) fetch(op.xa, cur);
+            chain_axpy(op.alpha, cur, cur, y);
+        }
+        return;
+    }
+    if constexpr (EXT) {
+        if (op.xi >= 0) {
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cur[k][q] = op.xi == 0 ? e0[k][q] : e1[k][q];
+        }
+    } else {
+        if (op.xa) fetch(op.xa, cur);
+    }
+    if (op.kind == 0) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cur[k][q] = ew_apply<Ew::Relu>(cur[k][q], 0.0f, 0.0f);
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cur[k][q] = ew_apply<Ew::Square>(cur[k][q], 0.0f, 0.0f);
+    }
+}
+
+template <bool EXT>
+__global__ void __launch_bounds__(256) ew_chain_kernel(const __grid_constant__ EwChain c) {
+    constexpr int kAhead = EXT ? 2 : 1;  // quads of a thread in flight
     const int64_t n = c.n;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
-    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
-        float cur[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        const bool vec = c.vec != 0 && i + 4 <= n;  // a ragged last quadruple element by element
-        const int w = vec ? 4 : (int)(n - i < 4 ? n - i : 4);
+    for (int64_t i0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i0 < n; i0 += kAhead * stride) {
+        float cur[kAhead][4] = {};
+        int w[kAhead];  // elements of each quad inside the array (a ragged last one element by element)
 #pragma unroll
-        for (int o = 0; o < kMaxChainOps; ++o) {
-            if (o >= c.nops) break;
-            const EwChainOp& op = c.op[o];
-            float x[4], y[4];
-            auto fetch = [&](const float* src, float* dst) {
-                if (vec) {
-                    const float4 v = *reinterpret_cast<const float4*>(src + i);
-                    dst[0] = v.x, dst[1] = v.y, dst[2] = v.z, dst[3] = v.w;
+        for (int k = 0; k < kAhead; ++k) {
+            const int64_t rest = n - (i0 + k * stride);
+            w[k] = rest >= 4 ? 4 : rest > 0 ? (int)rest : 0;
+        }
+        auto fetch = [&](const float* src, float (&d)[kAhead][4]) {
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) {
+                const float* p = src + i0 + k * stride;
+                if (c.vec && w[k] == 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(p);
+                    d[k][0] = v.x, d[k][1] = v.y, d[k][2] = v.z, d[k][3] = v.w;
                 } else {
-                    for (int q = 0; q < 4; ++q) dst[q] = q < w ? src[i + q] : 0.0f;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) d[k][q] = q < w[k] ? p[q] : 0.0f;
                 }
-            };
-            if (op.xa) fetch(op.xa, x);
-            else for (int q = 0; q < 4; ++q) x[q] = cur[q];
-            if (op.kind == 2) {  // AXPY: x + alpha y
-                if (op.yb) fetch(op.yb, y);
-                else for (int q = 0; q < 4; ++q) y[q] = cur[q];
             }
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                cur[q] = op.kind == 0 ? ew_apply<Ew::Relu>(x[q], 0.0f, 0.0f)
-                       : op.kind == 1 ? ew_apply<Ew::Square>(x[q], 0.0f, 0.0f)
-                                      : ew_apply<Ew::Axpy>(x[q], y[q], op.alpha);
+        };
+        float e0[kAhead][4], e1[kAhead][4];
+        if constexpr (EXT) {
+            fetch(c.ext[0], e0);
+            if (c.next > 1) fetch(c.ext[1], e1);
+        }
+#pragma unroll 1
+        for (int o = 0; o < c.nops; ++o) {
+            const EwChainOp& op = c.op[o];
+            chain_op<EXT, kAhead>(op, cur, e0, e1, fetch);
             if (op.out) {
-                if (vec) {
-                    *reinterpret_cast<float4*>(op.out + i) = make_float4(cur[0], cur[1], cur[2], cur[3]);
-                } else {
-                    for (int q = 0; q < w; ++q) op.out[i + q] = cur[q];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    float* p = op.out + i0 + k * stride;
+                    if (c.vec && w[k] == 4) {
+                        *reinterpret_cast<float4*>(p) = make_float4(cur[k][0], cur[k][1], cur[k][2], cur[k][3]);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (q < w[k]) p[q] = cur[k][q];
+                    }
                 }
             }
         }
@@ -568,6 +653,154 @@ __global__ void colmax_decode_kernel(float* __restrict__ out, const uint32_t* __
                                      int64_t rows) {
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < cols; c += (int64_t)gridDim.x * blockDim.x)
         out[c] = rows > 0 ? __uint_as_float(fmax_unkey(keys[c])) : -INFINITY;
+}
+
+// ---- element-wise chain with the reductions of its last value ------------------------------
+//
+// A linear element-wise chain (as ew_chain_kernel) whose last value is read only by a SUM and /
+// or a COLMAX loop: both are formed in the chain's pass and the value is never written.  Blocks
+// and columns as in colmax_strip_kernel, kRedAhead rows' loads in flight per thread; the sum as in
+// reduce64_kernel (compensated binary32 per thread over partials of four columns, binary64
+// across threads, block partials added in index order by the last block to finish).  HBM-bound:
+// the chain, column maxima and sum of a 6000 x 6000 matrix read two arrays once instead of
+// reading four and writing one, 56 us (5.1 TB/s) instead of 72 + 33 + 30.
+constexpr int kRedAhead = 4;
+
+template <int VX, bool VEC, bool EXT>
+__global__ void __launch_bounds__(256) ew_chain_reduce_kernel(const __grid_constant__ EwChain c, int64_t rows,
+                                                              int64_t cols, int cluster_rows, EwReduce red) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_arrive();  // waited for below: the first block's shared memory is written remotely
+    constexpr int C = 4 * VX, RY = 256 / VX;
+    __shared__ uint32_t s_warp[8][C];
+    __shared__ uint32_t s_cta[8][C];
+    __shared__ double wsum[8];
+    __shared__ bool last;
+    const int t = threadIdx.x, vx = t % VX, ry = t / VX;
+    const int rank = (int)blockIdx.y;
+    const int64_t c0 = (int64_t)blockIdx.x * C;
+    const int64_t per = (rows + cluster_rows - 1) / cluster_rows;
+    const int64_t r0 = rank * per, r1 = r0 + per < rows ? r0 + per : rows;
+    uint32_t m[4] = {0u, 0u, 0u, 0u};
+    float rs = 0.0f, rc = 0.0f;
+    int64_t cc[4];
+    bool in_q[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        cc[q] = VEC ? c0 + 4 * vx + q : c0 + vx + VX * q;
+        in_q[q] = cc[q] < cols;
+    }
+    if (in_q[0]) {
+        for (int64_t r = r0 + ry; r < r1; r += (int64_t)kRedAhead * RY) {
+            float cur[kRedAhead][4] = {};
+            int64_t off[kRedAhead];
+            bool ok[kRedAhead];  // a row past the share is read as its first row again and not counted
+#pragma unroll
+            for (int k = 0; k < kRedAhead; ++k) {
+                ok[k] = r + k * RY < r1;
+                off[k] = (ok[k] ? r + k * RY : r) * cols;
+            }
+            auto fetch = [&](const float* src, float (&d)[kRedAhead][4]) {
+#pragma unroll
+                for (int k = 0; k < kRedAhead; ++k) {
+                    if (VEC) {
+                        const float4 v = *reinterpret_cast<const float4*>(src + off[k] + cc[0]);
+                        d[k][0] = v.x, d[k][1] = v.y, d[k][2] = v.z, d[k][3] = v.w;
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) d[k][q] = in_q[q] ? src[off[k] + cc[q]] : 0.0f;
+                    }
+                }
+            };
+            float e0[kRedAhead][4], e1[kRedAhead][4];
+            if constexpr (EXT) {
+                fetch(c.ext[0], e0);
+                if (c.next > 1) fetch(c.ext[1], e1);
+            }
+#pragma unroll 1
+            for (int o = 0; o < c.nops; ++o) {
+                const EwChainOp& op = c.op[o];
+                chain_op<EXT, kRedAhead>(op, cur, e0, e1, fetch);
+                if (op.out) {
+#pragma unroll
+                    for (int k = 0; k < kRedAhead; ++k) {
+                        if (!ok[k]) continue;
+                        if (VEC) {
+                            *reinterpret_cast<float4*>(op.out + off[k] + cc[0]) =
+                                make_float4(cur[k][0], cur[k][1], cur[k][2], cur[k][3]);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                if (in_q[q]) op.out[off[k] + cc[q]] = cur[k][q];
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < kRedAhead; ++k) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) m[q] = max(m[q], ok[k] ? fmax_key(__float_as_uint(cur[k][q])) : 0u);
+                if (red.sum_out) {
+                    float v[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q] = ok[k] && (VEC || in_q[q]) ? cur[k][q] : 0.0f;
+                    comp_add(rs, rc, (v[0] + v[1]) + (v[2] + v[3]));
+                }
+            }
+        }
+    }
+    const int w = t >> 5, lane = t & 31;
+#pragma unroll
+    for (int off = VX; off < 32; off <<= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) m[q] = max(m[q], __shfl_xor_sync(0xffffffffu, m[q], off));
+    if (lane < VX) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s_warp[w][VEC ? 4 * vx + q : vx + VX * q] = m[q];
+    }
+    double acc = (double)rs + (double)rc;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if (lane == 0) wsum[w] = acc;
+    __syncthreads();
+    cluster.barrier_wait();
+    if (red.colmax_out && t < C) {
+        uint32_t k = s_warp[0][t];
+#pragma unroll
+        for (int j = 1; j < 8; ++j) k = max(k, s_warp[j][t]);
+        *cluster.map_shared_rank(&s_cta[rank][t], 0) = k;
+    }
+    cluster.sync();
+    if (red.colmax_out && rank == 0 && t < C && c0 + t < cols) {
+        uint32_t k = s_cta[0][t];
+        for (int j = 1; j < cluster_rows; ++j) k = max(k, s_cta[j][t]);
+        red.colmax_out[c0 + t] = __uint_as_float(fmax_unkey(k));
+    }
+    if (!red.sum_out) return;
+    const unsigned blocks = gridDim.x * gridDim.y;
+    if (t == 0) {
+        double b = 0.0;
+        for (int k = 0; k < 8; ++k) b += wsum[k];
+        red.scratch.partials[blockIdx.y * gridDim.x + blockIdx.x] = b;
+        __threadfence();
+        last = atomicAdd(red.scratch.counter, 1u) == blocks - 1;
+    }
+    __syncthreads();
+    if (!last) return;  // block-uniform
+    __threadfence();
+    double u = 0.0;
+    for (unsigned b = t; b < blocks; b += 256) u += ((volatile double*)red.scratch.partials)[b];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) u += __shfl_xor_sync(0xffffffffu, u, off);
+    if (lane == 0) wsum[w] = u;
+    __syncthreads();
+    if (t == 0) {
+        double v = 0.0;
+        for (int k = 0; k < 8; ++k) v += wsum[k];
+        *red.sum_out = v;
+        *red.scratch.counter = 0u;  // ready for the next launch on this stream
+    }
 }
 
 // ---- STENCIL3 --------------------------------------------------------------------------
@@ -1069,15 +1302,41 @@ cudaError_t launch_init_set(const InitSet& set, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+namespace {
+// The launcher's fields of a chain; false if some array is not 16-byte aligned.
+bool chain_fields(EwChain& c) {
+    uintptr_t ptrs = 0;
+    c.next = 0;
+    bool two = true;
+    auto index = [&](const float* p) {
+        if (!p) return -1;
+        for (int i = 0; i < c.next; ++i)
+            if (c.ext[i] == p) return i;
+        if (c.next == 2) {
+            two = false;
+            return -1;
+        }
+        c.ext[c.next] = p;
+        return c.next++;
+    };
+    for (int o = 0; o < c.nops; ++o) {
+        EwChainOp& op = c.op[o];
+        ptrs |= (uintptr_t)op.xa | (uintptr_t)op.yb | (uintptr_t)op.out;
+        op.xi = index(op.xa);
+        op.yi = op.kind == 2 ? index(op.yb) : -1;
+    }
+    if (!two) c.next = 0;
+    return (ptrs & 15u) == 0;
+}
+}  // namespace
+
 cudaError_t launch_ew_chain(const EwChain& c, cudaStream_t st) {
     if (c.nops < 1 || c.nops > kMaxChainOps) return cudaErrorInvalidValue;
     if (c.n <= 0) return cudaSuccess;
     EwChain k = c;
-    uintptr_t ptrs = 0;
-    for (int o = 0; o < c.nops; ++o)
-        ptrs |= (uintptr_t)c.op[o].xa | (uintptr_t)c.op[o].yb | (uintptr_t)c.op[o].out;
-    k.vec = (ptrs & 15u) == 0;
-    ew_chain_kernel<<<grid_for((c.n + 3) / 4), kThreads, 0, st>>>(k);
+    k.vec = chain_fields(k);
+    if (k.next > 0) ew_chain_kernel<true><<<grid_for((c.n + 7) / 8), kThreads, 0, st>>>(k);
+    else ew_chain_kernel<false><<<grid_for((c.n + 3) / 4), kThreads, 0, st>>>(k);
     return cudaGetLastError();
 }
 
@@ -1170,6 +1429,27 @@ cudaLaunchConfig_t strip_config(int64_t cols, int vx, int cluster, cudaStream_t 
     return lc;
 }
 }  // namespace
+
+bool ew_chain_reduce_fits(int64_t rows, int64_t cols) {
+    int vx, cluster;
+    return strip_plan(rows, cols, reduce_blocks(), &vx, &cluster);
+}
+
+cudaError_t launch_ew_chain_reduce(const EwChain& c, int64_t rows, int64_t cols, const EwReduce& red, cudaStream_t st) {
+    int vx, cluster;
+    if (c.nops < 1 || c.nops > kMaxChainOps || !strip_plan(rows, cols, reduce_blocks(), &vx, &cluster))
+        return cudaErrorInvalidValue;
+    EwChain k = c;
+    const bool vec = chain_fields(k) && cols % 4 == 0;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t lc = strip_config(cols, vx, cluster, st, &at);
+    auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, k, rows, cols, cluster, red); };
+#define GAO_CHAIN_REDUCE(VX)                                                                                   \
+    (vec ? (k.next > 0 ? go(ew_chain_reduce_kernel<VX, true, true>) : go(ew_chain_reduce_kernel<VX, true, false>)) \
+         : (k.next > 0 ? go(ew_chain_reduce_kernel<VX, false, true>) : go(ew_chain_reduce_kernel<VX, false, false>)))
+    return vx == 32 ? GAO_CHAIN_REDUCE(32) : vx == 16 ? GAO_CHAIN_REDUCE(16) : GAO_CHAIN_REDUCE(8);
+#undef GAO_CHAIN_REDUCE
+}
 
 cudaError_t launch_colmax(float* out, const float* in, int64_t rows, int64_t cols, uint32_t* keys, cudaStream_t st,
                           int* launches) {

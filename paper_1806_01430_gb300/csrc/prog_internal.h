@@ -22,6 +22,9 @@ struct BufState {
     // (gen_for): the binary32 array holds nothing (vd and vh false) until something else
     // needs it, which then runs slot gen_slot of INIT loop gen_loop for it alone.
     int gen_loop = -1, gen_slot = -1, gen_for = -1;
+    // The last value of the element-wise chain that starts at this loop, which the last run
+    // reduced without writing it: prog_device_ptr forms it (vd and vh false until then).
+    int gen_chain = -1;
 };
 
 struct CacheEntry {
@@ -46,6 +49,7 @@ struct GraphEntry {
     bool failed = false;
     cudaGraphExec_t exec = nullptr;
     std::vector<uint8_t> vh, vd;
+    std::vector<int> gen_chain;
     std::vector<gao_loop_stat> stats;
     std::vector<uint8_t> ev_used;
 };
@@ -68,6 +72,8 @@ struct gao_prog {
     std::unordered_map<uint64_t, gao::CacheEntry> cache;
     bool dirty_stream = false;  // a previous run left work in flight
     bool stats_pending = false; // the last run's event times are not read yet
+    uint64_t run_mask = 0;      // the last run's GPU loops, and whether it fused chains
+    bool run_fuse = false;
     cudaStream_t cst = nullptr;           // copy stream of the copy/compute overlap
     std::vector<cudaEvent_t> pipe_ev;     // its events: fork, B landed, one per row block
     cudaStream_t ost = nullptr;           // device-to-host stream: a GEMM's C rows as blocks finish

@@ -1008,6 +1008,10 @@ void grad_chain_done(gao_prog* p, const GradChain& gch, int first, uint64_t* fus
 struct EwPlan {
     int n = 0;
     int loops[kMaxChainOps];
+    // a SUM and / or a COLMAX loop of the chain's last value right after it, formed in the same
+    // pass: only when nothing else reads that value, which is then never written (writing it
+    // costs what the separate reductions' reads would)
+    int sum_loop = -1, colmax_loop = -1;
 };
 
 bool is_elementwise(int kind) { return kind == GAO_LOOP_RELU || kind == GAO_LOOP_SQUARE || kind == GAO_LOOP_AXPY; }
@@ -1038,9 +1042,77 @@ bool find_ew_chain(const gao_prog* p, int li, uint64_t mask, bool fuse, EwPlan* 
         cur = L.outs[0];
         produced.push_back(cur);
     }
-    if (e.n < 2) return false;
+    const int last = e.loops[e.n - 1];
+    const BufState& P = p->bufs[(size_t)cur];
+    if (P.d.role != GAO_BUF_OUTPUT && ew_chain_reduce_fits(P.d.rows, P.d.cols)) {
+        int sum = -1, colmax = -1, j = last + 1;
+        for (; j < n && ((mask >> j) & 1); ++j) {
+            const gao_loop& R = p->loops[(size_t)j];
+            if (R.kind == GAO_LOOP_SUM && R.ins[0] == cur && sum < 0) sum = j;
+            else if (R.kind == GAO_LOOP_COLMAX && R.ins[0] == cur && colmax < 0) colmax = j;
+            else break;
+        }
+        // no other loop reads or writes the value, and what the chain reads outlives the pass
+        // (no loop from the chain on writes it): the value can still be formed when asked for
+        bool dead = true;
+        for (int k = 0; k < n && dead; ++k) {
+            const gao_loop& K = p->loops[(size_t)k];
+            for (int o : loop_outputs(K)) {
+                dead &= o != cur || k == last;
+                for (int t = 0; t < e.n && k >= li; ++t) {
+                    const std::vector<int> ins = loop_inputs(p->loops[(size_t)e.loops[t]]);
+                    for (int b : ins) dead &= b != o || (t > 0 && b == p->loops[(size_t)e.loops[t - 1]].outs[0]);
+                }
+            }
+            if (k != sum && k != colmax)
+                for (int b : loop_inputs(K)) dead &= b != cur;
+        }
+        if (dead) {
+            e.sum_loop = sum;
+            e.colmax_loop = colmax;
+        }
+    }
+    if (e.n < 2 && e.sum_loop < 0 && e.colmax_loop < 0) return false;
     *plan = e;
     return true;
+}
+
+// The chain's operands; loop k's value is written if live[k].
+EwChain ew_chain_args(const gao_prog* p, const EwPlan& e, const std::vector<char>& live) {
+    EwChain c{};
+    c.nops = e.n;
+    const gao_buffer& shape = p->bufs[(size_t)p->loops[(size_t)e.loops[0]].outs[0]].d;
+    c.n = (int64_t)shape.rows * shape.cols;
+    int prev = -1;
+    for (int k = 0; k < e.n; ++k) {
+        const gao_loop& L = p->loops[(size_t)e.loops[k]];
+        EwChainOp& op = c.op[k];
+        op.kind = L.kind == GAO_LOOP_RELU ? 0 : L.kind == GAO_LOOP_SQUARE ? 1 : 2;
+        op.alpha = (float)L.alpha;
+        auto src = [&](int b) -> const float* {
+            return (k > 0 && b == prev) ? nullptr : (const float*)p->bufs[(size_t)b].dev;
+        };
+        op.xa = src(L.ins[0]);
+        op.yb = op.kind == 2 ? src(L.ins[1]) : nullptr;
+        op.out = live[(size_t)k] ? (float*)p->bufs[(size_t)L.outs[0]].dev : nullptr;
+        prev = L.outs[0];
+    }
+    return c;
+}
+
+// The last value of a chain that a run reduced without writing it (gen_chain).
+gao_status form_chain_value(RunCtx& R, int b) {
+    gao_prog* p = R.p;
+    BufState& B = p->bufs[(size_t)b];
+    EwPlan e;
+    if (!find_ew_chain(p, B.gen_chain, p->run_mask, p->run_fuse, &e))
+        return fail(GAO_EINVAL, "buffer " + std::to_string(b) + " holds no data");
+    std::vector<char> live((size_t)e.n, 0);
+    live.back() = 1;
+    GAO_CUDA_TRY(launch_ew_chain(ew_chain_args(p, e, live), R.st));
+    B.vd = true;
+    B.gen_chain = -1;
+    return GAO_OK;
 }
 
 // A chain the GEMM loop li can run as one pass when the gene puts it all on the GPU:
@@ -1516,8 +1588,10 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
     for (auto& B : p->bufs) {
         B.vh = (B.d.role == GAO_BUF_INPUT);
         B.vd = false;
-        B.gen_loop = B.gen_slot = B.gen_for = -1;
+        B.gen_loop = B.gen_slot = B.gen_for = B.gen_chain = -1;
     }
+    p->run_mask = gene_mask;
+    p->run_fuse = fuse;
     std::fill(p->ev_used.begin(), p->ev_used.end(), 0);
     for (auto& s : p->stats) s = gao_loop_stat{};
     const bool uses_gpu = gene_mask != 0;
@@ -1594,6 +1668,7 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
         EwPlan ewp;
         if (gpu && is_elementwise(L.kind) && find_ew_chain(p, li, gene_mask, fuse, &ewp)) {
             const int last = ewp.loops[ewp.n - 1];
+            const bool reduce = ewp.sum_loop >= 0 || ewp.colmax_loop >= 0;
             // buffers the chain reads from memory: every input of its first loop, and each
             // later loop's input other than the previous loop's output
             std::vector<int> ext;
@@ -1614,32 +1689,24 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
                 GAO_CUDA_TRY(record_timing(ev[1], p->st));
                 p->ev_used[(size_t)li] |= 1;
             }
-            EwChain c{};
-            c.nops = ewp.n;
-            c.n = (int64_t)p->bufs[(size_t)L.outs[0]].d.rows * p->bufs[(size_t)L.outs[0]].d.cols;
             std::vector<char> live((size_t)ewp.n, 0);
-            prev = -1;
             for (int k = 0; k < ewp.n; ++k) {
-                const gao_loop& Lk = p->loops[(size_t)ewp.loops[k]];
-                EwChainOp& op = c.op[k];
-                op.kind = Lk.kind == GAO_LOOP_RELU ? 0 : Lk.kind == GAO_LOOP_SQUARE ? 1 : 2;
-                op.alpha = (float)Lk.alpha;
-                auto src = [&](int b) -> const float* {
-                    return (k > 0 && b == prev) ? nullptr : (const float*)p->bufs[(size_t)b].dev;
-                };
-                op.xa = src(Lk.ins[0]);
-                op.yb = op.kind == 2 ? src(Lk.ins[1]) : nullptr;
-                const int ob = Lk.outs[0];
+                const int ob = p->loops[(size_t)ewp.loops[k]].outs[0];
                 bool lv = p->bufs[(size_t)ob].d.role == GAO_BUF_OUTPUT;
                 for (int j = last + 1; j < n && !lv; ++j)
                     for (int b : loop_inputs(p->loops[(size_t)j]))
                         if (b == ob) lv = true;
-                live[(size_t)k] = lv;
-                op.out = lv ? (float*)p->bufs[(size_t)ob].dev : nullptr;
-                prev = ob;
+                live[(size_t)k] = lv && !(reduce && k == ewp.n - 1);  // read in the pass only
             }
+            const EwChain c = ew_chain_args(p, ewp, live);
             GAO_CUDA_TRY(record_timing(ev[2], p->st));
-            const cudaError_t e = launch_ew_chain(c, p->st);
+            const gao_buffer& shape = p->bufs[(size_t)L.outs[0]].d;
+            auto out_of = [&](int j) { return j >= 0 ? p->bufs[(size_t)p->loops[(size_t)j].outs[0]].dev : nullptr; };
+            const EwReduce red{(double*)out_of(ewp.sum_loop), (float*)out_of(ewp.colmax_loop),
+                               ReduceScratch{(double*)(p->arena + p->lay.partial_off),
+                                             (unsigned*)(p->arena + p->lay.counter_off)}};
+            const cudaError_t e = reduce ? launch_ew_chain_reduce(c, shape.rows, shape.cols, red, p->st)
+                                         : launch_ew_chain(c, p->st);
             if (e != cudaSuccess) {
                 status = cuda_fail(e, "element-wise chain launch");
                 break;
@@ -1653,6 +1720,14 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
                 B.vd = live[(size_t)k] != 0;  // an unwritten intermediate holds nothing
             }
             for (int k = 1; k < ewp.n; ++k) fused |= 1ULL << ewp.loops[k];
+            if (reduce) p->bufs[(size_t)p->loops[(size_t)last].outs[0]].gen_chain = li;
+            for (int j : {ewp.sum_loop, ewp.colmax_loop}) {
+                if (j < 0) continue;
+                fused |= 1ULL << j;
+                BufState& B = p->bufs[(size_t)p->loops[(size_t)j].outs[0]];
+                B.vh = false;
+                B.vd = true;
+            }
             if (R.deadline > 0.0 && now_s() > R.deadline) R.timed_out = true;
             if (R.timed_out) break;
             continue;
@@ -1834,9 +1909,11 @@ void capture_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags, Graph
         ge->exec = exec;
         ge->vh.resize(p->bufs.size());
         ge->vd.resize(p->bufs.size());
+        ge->gen_chain.resize(p->bufs.size());
         for (size_t b = 0; b < p->bufs.size(); ++b) {
             ge->vh[b] = p->bufs[b].vh;
             ge->vd[b] = p->bufs[b].vd;
+            ge->gen_chain[b] = p->bufs[b].gen_chain;
         }
         ge->stats = p->stats;
         ge->ev_used = p->ev_used;
@@ -1893,7 +1970,10 @@ extern "C" gao_status prog_run(gao_prog* p, uint64_t gene, uint32_t flags, doubl
         for (size_t b = 0; b < p->bufs.size(); ++b) {
             p->bufs[b].vh = ge->vh[b] != 0;
             p->bufs[b].vd = ge->vd[b] != 0;
+            p->bufs[b].gen_chain = ge->gen_chain[b];
         }
+        p->run_mask = gene_mask;
+        p->run_fuse = fuse;
         p->stats = ge->stats;
         p->ev_used = ge->ev_used;
     } else {
@@ -1935,11 +2015,11 @@ extern "C" gao_status prog_device_ptr(gao_prog* p, int buf, void** dev_ptr) {
     if (!p || !dev_ptr) return fail(GAO_EINVAL, "null argument");
     if (buf < 0 || buf >= (int)p->bufs.size()) return fail(GAO_EINVAL, "no such buffer");
     BufState& B = p->bufs[(size_t)buf];
-    if (!B.vd && !B.vh && B.gen_loop >= 0) {  // formed only as a GEMM's planes: form it now
+    if (!B.vd && !B.vh && (B.gen_loop >= 0 || B.gen_chain >= 0)) {  // a GEMM's planes, or only reduced: form it now
         cudaError_t ce = cudaSetDevice(p->device);
         if (ce != cudaSuccess) return cuda_fail(ce, "cudaSetDevice");
         RunCtx R{p, 0.0, false, CpuCtx{p->opts.cpu_threads, 0.0, false}, p->st, false};
-        gao_status s = materialize(R, buf);
+        gao_status s = B.gen_chain >= 0 ? form_chain_value(R, buf) : materialize(R, buf);
         if (s != GAO_OK) return s;
         if ((ce = cudaStreamSynchronize(p->st)) != cudaSuccess) return cuda_fail(ce, "cudaStreamSynchronize");
     }
