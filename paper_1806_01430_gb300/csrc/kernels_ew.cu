@@ -1005,35 +1005,72 @@ __global__ void __launch_bounds__(kStencilThreads, CHAIN ? kChainBlocks : 8)
 // The image program's first stencil P0 (the blur, B = P0(X)) and the gradient chain on its
 // output (g1 = P1(B), g2 = P2(B), their squares, m = s1 + alpha s2, and with RED the sum and
 // column maxima of m), formed in one pass over the raw image X.  Each thread walks down a
-// strip of rows holding two raw rows and three rows of B in registers: at output row r it
-// forms B's row r + 1 from raw rows r .. r + 2 and the chain's row r from B's rows r - 1 ..
-// r + 1, so neither B nor the chain's intermediates go through memory (B is written only when
-// something else reads it).  B is zero outside the image, as the separate loops pad it, and
-// every value is formed with the separate loops' operations, so the bits are theirs.
-// Lanes hold kEdgeNC (eight) columns each; lanes 1 .. 30 of a warp produce its 240 output
-// columns, and lanes 0 and 31 hold the eight columns either side, whose raw values and B
-// values their neighbours take by shuffle, so no lane loads an edge column of its own.
-constexpr int kEdgeNC = 8;          // columns a lane holds (a multiple of 4)
+// strip of rows holding two raw rows and two rows of B in registers: at output row r it forms
+// B's row r + 1 from raw rows r .. r + 2 and the chain's row r from B's rows r - 1 .. r + 1, so
+// neither B nor the chain's intermediates go through memory (B is written only when something
+// else reads it).  B is zero outside the image, as the separate loops pad it, and every value
+// is formed with the separate loops' operations, so the bits are theirs.
+// Lanes hold eight columns each; lanes 1 .. 30 of a warp produce its 240 output columns, and
+// lanes 0 and 31 hold the eight columns either side, whose raw values and B values their
+// neighbours take by shuffle, so no lane loads an edge column of its own.
+//
+// What bounds it: instruction issue, not HBM (one read of X, nothing written but the outputs
+// asked for).  So the arithmetic is packed (fma / add / mul.rn.f32x2: two columns an
+// instruction, the same rounding each): a row is held as the pairs (x_k, x_k+4), k = -1 .. 4,
+// in which a stencil's left and right neighbours are the neighbouring pairs as they are, where
+// pairs of adjacent columns would have to be rebuilt for every odd shift.  Rows are walked
+// three at a time, so that the three-row windows rotate by name and not by moves.
+// 8192 x 8192: 84 us; 107 with a column an instruction, moves and a second, part-filled wave.
+constexpr int kEdgeNC = 8;               // columns a lane holds
 constexpr int kEdgeCols = 30 * kEdgeNC;  // output columns of a warp (lanes 1 .. 30)
-constexpr int kEdgeBlocks = 5;      // resident 128-thread blocks per SM the kernel is built for
-constexpr int kEdgeAhead = 1;       // raw rows of loads in flight
+constexpr int kEdgeBlocks = 4;           // resident 128-thread blocks per SM the kernel is built for
 constexpr int kEdgeBlockCols = kEdgeCols * (kStencilThreads / 32);  // output columns of a block
 
-// A lane's columns c0 .. c0 + kEdgeNC - 1 of one raw row (zero outside the image): with 16-byte
-// rows, groups of four that are each wholly inside or outside the image.
-struct EdgeRow {
-    float4 g[kEdgeNC / 4];
+using f32x2 = unsigned long long;  // two binary32 values, the first in the low half
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// A row as a lane holds it: p[k + 1] = (x_k, x_k+4) of its columns c0 + k, k = -1 .. 4.
+struct EdgePairs {
+    f32x2 p[6];
 };
 
+// The eight columns c0 .. c0 + 7 of a lane as loaded (g[0] the first four).
+struct EdgeRow {
+    float4 g[2];
+};
+
+// p: row y's first column of the lane (any value when the row is outside the image).
 template <bool VEC>
-__device__ __forceinline__ void edge_load(EdgeRow& r, const float* __restrict__ in, int64_t y, int64_t ylim,
-                                          int64_t cols, int64_t c0, const bool inc[kEdgeNC]) {
+__device__ __forceinline__ void edge_load(EdgeRow& r, const float* __restrict__ p, bool row_in, const bool inc[kEdgeNC]) {
+    r.g[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    r.g[1] = r.g[0];
+    if (!row_in) return;
 #pragma unroll
-    for (int k = 0; k < kEdgeNC / 4; ++k) r.g[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (y < 0 || y >= ylim) return;
-    const float* p = in + y * cols + c0;
-#pragma unroll
-    for (int k = 0; k < kEdgeNC / 4; ++k) {
+    for (int k = 0; k < 2; ++k) {
         if (VEC) {
             if (inc[4 * k]) r.g[k] = __ldg(reinterpret_cast<const float4*>(p + 4 * k));
         } else {
@@ -1045,38 +1082,56 @@ __device__ __forceinline__ void edge_load(EdgeRow& r, const float* __restrict__ 
     }
 }
 
-// The values c0 - 1 .. c0 + kEdgeNC of a row whose columns c0 .. c0 + kEdgeNC - 1 this lane
-// holds in b (the first and last lane's outer values are not used).
-__device__ __forceinline__ void edge_spread(float v[kEdgeNC + 2], const float b[kEdgeNC]) {
-    v[0] = __shfl_up_sync(0xffffffffu, b[kEdgeNC - 1], 1);
-#pragma unroll
-    for (int q = 0; q < kEdgeNC; ++q) v[q + 1] = b[q];
-    v[kEdgeNC + 1] = __shfl_down_sync(0xffffffffu, b[0], 1);
+// The pairs of a row from the lane's own four (p[1] .. p[4] set): the columns either side come
+// from the neighbouring lanes (the first and last lane's outer values are not used).
+__device__ __forceinline__ void edge_spread(EdgePairs& r) {
+    const float2 first = unpack2(r.p[1]), last = unpack2(r.p[4]);
+    r.p[0] = pack2(__shfl_up_sync(0xffffffffu, last.y, 1), last.x);     // (x_-1, x_3)
+    r.p[5] = pack2(first.y, __shfl_down_sync(0xffffffffu, first.x, 1)); // (x_4, x_8)
 }
 
-__device__ __forceinline__ void edge_flat(float b[kEdgeNC], const EdgeRow& r) {
-#pragma unroll
-    for (int k = 0; k < kEdgeNC / 4; ++k) {
-        b[4 * k] = r.g[k].x;
-        b[4 * k + 1] = r.g[k].y;
-        b[4 * k + 2] = r.g[k].z;
-        b[4 * k + 3] = r.g[k].w;
-    }
+__device__ __forceinline__ void edge_pairs(EdgePairs& r, const EdgeRow& v) {
+    r.p[1] = pack2(v.g[0].x, v.g[1].x);
+    r.p[2] = pack2(v.g[0].y, v.g[1].y);
+    r.p[3] = pack2(v.g[0].z, v.g[1].z);
+    r.p[4] = pack2(v.g[0].w, v.g[1].w);
+    edge_spread(r);
 }
 
 template <bool VEC>
-__device__ __forceinline__ void edge_store(float* row, int64_t c0, const bool outc[kEdgeNC], const float v[kEdgeNC]) {
+__device__ __forceinline__ void edge_store(float* row, int64_t c0, const bool outc[kEdgeNC], const f32x2 v[4]) {
+    float x[kEdgeNC];
 #pragma unroll
-    for (int k = 0; k < kEdgeNC / 4; ++k) {
+    for (int k = 0; k < 4; ++k) {
+        const float2 u = unpack2(v[k]);
+        x[k] = u.x;
+        x[k + 4] = u.y;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
         if (VEC) {
             if (outc[4 * k])
-                *reinterpret_cast<float4*>(row + c0 + 4 * k) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                *reinterpret_cast<float4*>(row + c0 + 4 * k) = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
         } else {
 #pragma unroll
             for (int q = 4 * k; q < 4 * k + 4; ++q)
-                if (outc[q]) row[c0 + q] = v[q];
+                if (outc[q]) row[c0 + q] = x[q];
         }
     }
+}
+
+// stencil9 on pair k of three rows: the same terms in the same order for both columns.
+template <int P>
+__device__ __forceinline__ f32x2 stencil9_pair(const StencilW& w, const EdgePairs& up, const EdgePairs& md,
+                                               const EdgePairs& dn, int k) {
+    const EdgePairs* rows[3] = {&up, &md, &dn};
+    f32x2 s = 0ull;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+        const float wt = P >= 0 ? stencil_preset(P, t) : w.w[t];
+        if (wt != 0.0f) s = fma2(pack2(wt, wt), rows[t / 3]->p[k + t % 3], s);
+    }
+    return s;
 }
 
 template <bool VEC, int P0, int P1, int P2, bool RED, bool STORE>
@@ -1102,112 +1157,113 @@ __global__ void __launch_bounds__(kStencilThreads, kEdgeBlocks)
     const int64_t r0 = row_begin + (int64_t)blockIdx.y * strip;
     const int64_t r1 = r0 + strip < row_end ? r0 + strip : row_end;
     const int64_t ylim = r1 + 2 < rows ? r1 + 2 : rows;
-    // B's row from the raw rows above, at and below it (zero outside the image)
     // a lane whose columns are all inside the image zeroes none of its B values but in the
     // rows above and below it, so it skips the per-value choice elsewhere
     bool all_in = true;
 #pragma unroll
     for (int q = 0; q < NC; ++q) all_in = all_in && inc[q];
-    auto blur = [&](float b[NC], const float* xu, const float* xm, const float* xd, bool row_in) {
+    // B's row from the raw rows above, at and below it (zero outside the image)
+    auto blur = [&](EdgePairs& b, const EdgePairs& xu, const EdgePairs& xm, const EdgePairs& xd, bool row_in) {
 #pragma unroll
-        for (int q = 0; q < NC; ++q) b[q] = stencil9<P0>(w0, xu, xm, xd, q);
+        for (int k = 0; k < 4; ++k) b.p[k + 1] = stencil9_pair<P0>(w0, xu, xm, xd, k);
         if (!(row_in && all_in)) {
 #pragma unroll
-            for (int q = 0; q < NC; ++q) b[q] = (row_in && inc[q]) ? b[q] : 0.0f;
+            for (int k = 0; k < 4; ++k) {
+                const float2 u = unpack2(b.p[k + 1]);
+                b.p[k + 1] = pack2(row_in && inc[k] ? u.x : 0.0f, row_in && inc[k + 4] ? u.y : 0.0f);
+            }
         }
     };
-    auto store_b = [&](int64_t y, const float b[NC]) {
-        if (STORE && bout && y >= r0 && y < r1) edge_store<VEC>(bout + y * cols, c0, outc, b);
+    auto store_b = [&](int64_t y, const EdgePairs& b) {
+        if (STORE && bout && y >= r0 && y < r1) edge_store<VEC>(bout + y * cols, c0, outc, b.p + 1);
     };
-    float xa[NC + 2], xb[NC + 2];  // raw rows r, r + 1
-    float ba[NC + 2], bb[NC + 2];  // B's rows r - 1, r
+    auto row_ptr = [&](int64_t y) { return in + y * cols + c0; };
+    auto load_row = [&](EdgeRow& v, int64_t y) { edge_load<VEC>(v, row_ptr(y), y >= 0 && y < ylim, inc); };
+    EdgePairs xa, xb, xc, ba, bb, bc;
     {
         EdgeRow v;
-        float x0[NC + 2], f[NC], t[NC];
-        edge_load<VEC>(v, in, r0 - 2, ylim, cols, c0, inc);
-        edge_flat(f, v);
-        edge_spread(x0, f);
-        edge_load<VEC>(v, in, r0 - 1, ylim, cols, c0, inc);
-        edge_flat(f, v);
-        edge_spread(xa, f);
-        edge_load<VEC>(v, in, r0, ylim, cols, c0, inc);
-        edge_flat(f, v);
-        edge_spread(xb, f);
-        blur(t, x0, xa, xb, r0 >= 1);  // B's row r0 - 1
-        edge_spread(ba, t);
-        edge_load<VEC>(v, in, r0 + 1, ylim, cols, c0, inc);
-        edge_flat(f, v);
-        edge_spread(x0, f);
-        blur(t, xa, xb, x0, r0 < rows);  // B's row r0
-        store_b(r0, t);
-        edge_spread(bb, t);
-#pragma unroll
-        for (int k = 0; k < NC + 2; ++k) {
-            xa[k] = xb[k];
-            xb[k] = x0[k];
-        }
+        EdgePairs x0;
+        load_row(v, r0 - 2);
+        edge_pairs(x0, v);
+        load_row(v, r0 - 1);
+        edge_pairs(xc, v);
+        load_row(v, r0);
+        edge_pairs(xa, v);
+        blur(ba, x0, xc, xa, r0 >= 1);  // B's row r0 - 1
+        edge_spread(ba);
+        load_row(v, r0 + 1);
+        edge_pairs(xb, v);
+        blur(bb, xc, xa, xb, r0 < rows);  // B's row r0
+        store_b(r0, bb);
+        edge_spread(bb);
     }
-    EdgeRow ring[kEdgeAhead];  // raw rows r + 2 .. r + 1 + kEdgeAhead, in flight
+    EdgeRow ring[3];  // raw rows row + 2 .. row + 4, in flight: one per step of the loop
 #pragma unroll
-    for (int k = 0; k < kEdgeAhead; ++k) edge_load<VEC>(ring[k], in, r0 + 2 + k, ylim, cols, c0, inc);
-    for (int64_t i = r0; i < r1; i += kEdgeAhead) {
+    for (int k = 0; k < 3; ++k) load_row(ring[k], r0 + 2 + k);
+    const float* pn = row_ptr(r0 + 5);
+    // output row `row`: raw rows row, row + 1 in x0, x1 and B's rows row - 1, row in b0, b1; raw
+    // row + 2 goes to x2 and B's row + 1 to b2
+    auto step = [&](int64_t row, EdgeRow& next, const EdgePairs& x0, const EdgePairs& x1, EdgePairs& x2, const EdgePairs& b0,
+                    const EdgePairs& b1, EdgePairs& b2) {
+        edge_pairs(x2, next);
+        edge_load<VEC>(next, pn, row + 5 < ylim, inc);
+        pn += cols;
+        blur(b2, x0, x1, x2, row + 1 < rows);
+        store_b(row + 1, b2);
+        edge_spread(b2);
+        f32x2 o[4], o2[4], a[4], b[4], m[4];
+        const f32x2 al = pack2(out.alpha, out.alpha);
 #pragma unroll
-        for (int k = 0; k < kEdgeAhead; ++k) {
-            const int64_t row = i + k;
-            if (row >= r1) break;  // block-uniform
-            float xn[NC + 2], bn[NC], bc[NC + 2], f[NC];
-            edge_flat(f, ring[k]);
-            edge_spread(xn, f);  // raw row + 2
-            edge_load<VEC>(ring[k], in, row + 2 + kEdgeAhead, ylim, cols, c0, inc);
-            blur(bn, xa, xb, xn, row + 1 < rows);  // B's row + 1
-            store_b(row + 1, bn);
-            edge_spread(bc, bn);
-            float o[NC], o2[NC], a[NC], b[NC], m[NC];
+        for (int k = 0; k < 4; ++k) {
+            o[k] = stencil9_pair<P1>(w1, b0, b1, b2, k);
+            o2[k] = stencil9_pair<P2>(w2, b0, b1, b2, k);
+            a[k] = mul2(o[k], o[k]);
+            b[k] = mul2(o2[k], o2[k]);
+            m[k] = out.swap ? fma2(al, a[k], b[k]) : fma2(al, b[k], a[k]);
+        }
+        if constexpr (STORE) {
+            const int64_t off = row * cols;
+            if (out.g1) edge_store<VEC>(out.g1 + off, c0, outc, o);
+            if (out.g2) edge_store<VEC>(out.g2 + off, c0, outc, o2);
+            if (out.s1) edge_store<VEC>(out.s1 + off, c0, outc, a);
+            if (out.s2) edge_store<VEC>(out.s2 + off, c0, outc, b);
+            if (out.m) edge_store<VEC>(out.m + off, c0, outc, m);  // null when only the reductions read m
+        }
+        if constexpr (RED) {
+            // the keys of every column are kept and only those of produced columns are raised at
+            // the end; the sum takes produced values only: with 16-byte rows a lane that produces
+            // none (the warp's outer lanes, lanes right of the image) sums values that are
+            // dropped at the end, and only the four columns right of the image in a lane that
+            // produces the other four are zeroed here
+            float v[NC];
 #pragma unroll
-            for (int q = 0; q < NC; ++q) {
-                o[q] = stencil9<P1>(w1, ba, bb, bc, q);
-                o2[q] = stencil9<P2>(w2, ba, bb, bc, q);
-                a[q] = __fmul_rn(o[q], o[q]);
-                b[q] = __fmul_rn(o2[q], o2[q]);
-                m[q] = out.swap ? __fmaf_rn(out.alpha, a[q], b[q]) : __fmaf_rn(out.alpha, b[q], a[q]);
+            for (int k = 0; k < 4; ++k) {
+                const float2 u = unpack2(m[k]);
+                v[k] = u.x;
+                v[k + 4] = u.y;
             }
-            if constexpr (STORE) {
-                const int64_t off = row * cols;
-                if (out.g1) edge_store<VEC>(out.g1 + off, c0, outc, o);
-                if (out.g2) edge_store<VEC>(out.g2 + off, c0, outc, o2);
-                if (out.s1) edge_store<VEC>(out.s1 + off, c0, outc, a);
-                if (out.s2) edge_store<VEC>(out.s2 + off, c0, outc, b);
-                if (out.m) edge_store<VEC>(out.m + off, c0, outc, m);  // null when only the reductions read m
-            }
-            if constexpr (RED) {
-                // the keys of every column are kept and only those of produced columns are
-                // raised at the end; the sum takes produced values only: with 16-byte rows a
-                // lane that produces none (the warp's outer lanes, lanes right of the image)
-                // sums values that are dropped at the end, and only the groups of four right
-                // of the image in a lane that produces some are zeroed here
 #pragma unroll
-                for (int q = 0; q < NC; ++q) mk[q] = max(mk[q], fmax_key(__float_as_uint(m[q])));
-                if (out.part) {
-                    float v[NC];
+            for (int q = 0; q < NC; ++q) mk[q] = max(mk[q], fmax_key(__float_as_uint(v[q])));
+            if (out.part) {
+                float t;
+                if (VEC) {
+                    const float2 g = unpack2(add2(add2(m[0], m[1]), add2(m[2], m[3])));
+                    t = g.x + (inc[4] ? g.y : 0.0f);
+                } else {
 #pragma unroll
-                    for (int q = 0; q < NC; ++q) v[q] = (VEC ? (q < 4 || inc[q]) : outc[q]) ? m[q] : 0.0f;
-                    float t = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < NC / 4; ++k) {
-                        const float g = (v[4 * k] + v[4 * k + 1]) + (v[4 * k + 2] + v[4 * k + 3]);
-                        t = k == 0 ? g : t + g;
-                    }
-                    comp_add(rs, rc, t);
+                    for (int q = 0; q < NC; ++q) v[q] = outc[q] ? v[q] : 0.0f;
+                    t = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
                 }
-            }
-#pragma unroll
-            for (int t = 0; t < NC + 2; ++t) {
-                xa[t] = xb[t];
-                xb[t] = xn[t];
-                ba[t] = bb[t];
-                bb[t] = bc[t];
+                comp_add(rs, rc, t);
             }
         }
+    };
+    for (int64_t row = r0; row < r1; row += 3) {  // block-uniform
+        step(row, ring[0], xa, xb, xc, ba, bb, bc);
+        if (row + 1 >= r1) break;
+        step(row + 1, ring[1], xb, xc, xa, bb, bc, ba);
+        if (row + 2 >= r1) break;
+        step(row + 2, ring[2], xc, xa, xb, bc, ba, bb);
     }
     if constexpr (RED) {
         if (out.keys && r1 > r0) {
@@ -1564,13 +1620,14 @@ cudaError_t launch_stencil_pass(const StencilOut& o, const float* in, int64_t ro
 }  // namespace
 
 namespace {
-// Grid of a blur + gradient-chain pass over `span` output rows: blocks of 480 output columns,
-// and strips of rows for two waves of the resident blocks, at least 16 rows per strip (each
-// strip reads four raw rows beyond its own).
+// Grid of a blur + gradient-chain pass over `span` output rows: blocks of 960 output columns, and
+// strips of rows for one wave of the resident blocks (each strip reads four raw rows beyond its
+// own and blurs two, so taller strips repeat less; a second wave would also start late), at
+// least 16 rows per strip.
+int64_t edge_strips(int64_t gx) { return std::max<int64_t>(1, (int64_t)sm_count() * kEdgeBlocks / gx); }
 void edge_grid(int64_t span, int64_t cols, int64_t* gx, int64_t* strip, int64_t* gy) {
     *gx = (cols + kEdgeBlockCols - 1) / kEdgeBlockCols;
-    const int64_t want_blocks = (int64_t)sm_count() * 2 * kEdgeBlocks;
-    const int64_t strips = (want_blocks + *gx - 1) / *gx;
+    const int64_t strips = edge_strips(*gx);
     int64_t s = (span + strips - 1) / strips;
     if (s < 16) s = 16;
     if ((span + s - 1) / s > 65535) s = (span + 65534) / 65535;
@@ -1591,8 +1648,7 @@ int64_t edge_chain_blocks(int64_t rows, int64_t cols) {
 int64_t edge_chain_blocks_max(int64_t cols) {
     if (cols <= 0) return 0;
     const int64_t gx = (cols + kEdgeBlockCols - 1) / kEdgeBlockCols;
-    const int64_t want_blocks = (int64_t)sm_count() * 2 * kEdgeBlocks;
-    return gx * ((want_blocks + gx - 1) / gx);
+    return gx * edge_strips(gx);
 }
 
 cudaError_t launch_edge_chain(const float* in, float* bout, int64_t rows, int64_t cols, int p0, int p1, int p2,
