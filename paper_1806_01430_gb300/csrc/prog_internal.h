@@ -99,6 +99,7 @@ struct RunCtx {
     CpuCtx cpu;
     cudaStream_t st;    // stream the GPU work and copies go to
     bool events;        // record per-loop CUDA events (not while capturing a graph)
+    bool out_pending = false;  // copies back queued on the third stream, not joined yet
 };
 
 gao_status make_valid(RunCtx& R, int b, bool on_gpu, gao_loop_stat& stat);

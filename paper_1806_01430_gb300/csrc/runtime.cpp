@@ -1416,7 +1416,13 @@ gao_status run_gpu_gemm_pipelined(RunCtx& R, int li, int64_t blocks, const Chain
 // are all in -- or, when the gene fuses the gradient chain on the stencil's output (gch,
 // from find_edge_chain), the blur and the chain in one pass form the rows whose five raw rows
 // are in.  A pixel is formed the same way whatever the row ranges, so the bits are those of
-// one launch.
+// one launch.  With early_out (the run copies its outputs back at its end), each frame-sized OUTPUT
+// that the pass writes and no loop from `after` on rewrites goes back to the host on a third
+// stream strip by strip, on the link's other direction while later strips are still coming in
+// (*on_host lists them).  The link bounds a 2160 x 3840 frame whose edge map is wanted back:
+// 66 MB both ways at ~210 GB/s in all are 316 us, and the pass takes 317 (402 with the map
+// copied back after the last strip).  The copies are joined into the program's stream by join_outputs, before
+// anything waits for that stream, so that later loops on the GPU do not wait for them.
 bool stencil_pipelined(const gao_prog* p, const gao_loop& L) {
     if (L.kind != GAO_LOOP_STENCIL3 || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT) return false;
     const BufState& X = p->bufs[(size_t)L.ins[0]];
@@ -1424,7 +1430,15 @@ bool stencil_pipelined(const gao_prog* p, const gao_loop& L) {
            L.ins[0] != L.outs[0];
 }
 
-gao_status run_gpu_stencil_pipelined(RunCtx& R, int li, const GradChain* gch) {
+// Whether two buffers' host memory overlaps.
+bool host_overlap(const gao_prog* p, int a, int b) {
+    const BufState &X = p->bufs[(size_t)a], &Y = p->bufs[(size_t)b];
+    const char *x = (const char*)X.host, *y = (const char*)Y.host;
+    return x && y && std::less<const char*>()(x, y + Y.bytes) && std::less<const char*>()(y, x + X.bytes);
+}
+
+gao_status run_gpu_stencil_pipelined(RunCtx& R, int li, const GradChain* gch, bool early_out, int after,
+                                     std::vector<int>* on_host) {
     gao_prog* p = R.p;
     const gao_loop& L = p->loops[(size_t)li];
     gao_loop_stat& S = p->stats[(size_t)li];
@@ -1434,6 +1448,26 @@ gao_status run_gpu_stencil_pipelined(RunCtx& R, int li, const GradChain* gch) {
     const int nb = kMaxRowBlocks;
     cudaStream_t st = R.st, cs = p->cst;
     cudaEvent_t* ev = &p->ev[(size_t)li * 6];
+    // the frame-sized outputs this pass writes
+    std::vector<int> written{L.outs[0]};
+    if (gch) {
+        written.clear();
+        if (gch->x_live) written.push_back(gch->x);
+        const int inter[4] = {gch->g1, gch->g2, gch->s1, gch->s2};
+        for (int t = 0; t < 4; ++t)
+            if (gch->live[t]) written.push_back(inter[t]);
+        if (gch->m_live) written.push_back(gch->m);
+    }
+    on_host->clear();
+    for (int b : written) {
+        bool back = early_out && p->bufs[(size_t)b].d.role == GAO_BUF_OUTPUT && p->bufs[(size_t)b].host;
+        for (size_t j = (size_t)after; j < p->loops.size() && back; ++j)
+            for (int o : loop_outputs(p->loops[j])) back &= o != b;
+        // bound host memory may be shared: an early copy must not land where a copy in still
+        // reads, or another output's copy writes
+        for (size_t k = 0; k < p->bufs.size() && back; ++k) back &= (int)k == b || !host_overlap(p, b, (int)k);
+        if (back) on_host->push_back(b);
+    }
     GAO_CUDA_TRY(cudaEventRecord(p->pipe_ev[0], st));  // the copy overwrites X on the device: after earlier work
     GAO_CUDA_TRY(cudaStreamWaitEvent(cs, p->pipe_ev[0], 0));
     GAO_CUDA_TRY(record_timing(ev[0], cs));
@@ -1457,6 +1491,23 @@ gao_status run_gpu_stencil_pipelined(RunCtx& R, int li, const GradChain* gch) {
     if (gch) red = grad_reduce_for(p, *gch);
     const bool reduce = gch && (gch->sum_loop >= 0 || gch->colmax_loop >= 0);
     int64_t formed = 0;  // output rows done
+    int sent = 0;        // copies back queued
+    auto send_rows = [&](int64_t f0, int64_t f1) -> gao_status {  // rows [f0, f1) of the outputs, as the pass leaves them
+        if (on_host->empty()) return GAO_OK;
+        R.out_pending = true;
+        cudaEvent_t done = p->out_ev[(size_t)sent++];
+        GAO_CUDA_TRY(cudaEventRecord(done, st));
+        GAO_CUDA_TRY(cudaStreamWaitEvent(p->ost, done, 0));
+        for (int b : *on_host) {
+            const BufState& Bo = p->bufs[(size_t)b];
+            const size_t off = (size_t)f0 * cols * 4, len = (size_t)(f1 - f0) * cols * 4;
+            GAO_CUDA_TRY(cudaMemcpyAsync((char*)Bo.host + off, Bo.dev + off, len, cudaMemcpyDeviceToHost, p->ost));
+            S.d2h_bytes += len;
+        }
+        GAO_CUDA_TRY(cudaEventRecord(p->out_ev[(size_t)kMaxRowBlocks], p->ost));
+        return GAO_OK;
+    };
+    gao_status sst = GAO_OK;
     for (int k = 0; k < nb; ++k) {
         GAO_CUDA_TRY(cudaStreamWaitEvent(st, p->pipe_ev[2 + (size_t)k], 0));
         if (!gch) {
@@ -1465,6 +1516,7 @@ gao_status run_gpu_stencil_pipelined(RunCtx& R, int li, const GradChain* gch) {
                 cudaError_t e = launch_stencil3(out, (const float*)X.dev, rows, cols, preset, st, formed, f1);
                 if (e != cudaSuccess) return cuda_fail(e, "stencil strip launch");
                 S.launches += 1;
+                if ((sst = send_rows(formed, f1)) != GAO_OK) return sst;
                 formed = f1;
             }
             continue;
@@ -1484,12 +1536,22 @@ gao_status run_gpu_stencil_pipelined(RunCtx& R, int li, const GradChain* gch) {
             if (e != cudaSuccess) return cuda_fail(e, "blur and gradient chain strip launch");
             S.launches += nl;
             red.part_at += edge_chain_blocks(f1 - formed, cols);
+            if ((sst = send_rows(formed, f1)) != GAO_OK) return sst;
             formed = f1;
         }
     }
     GAO_CUDA_TRY(record_timing(ev[3], st));
     X.vd = true;
     p->ev_used[(size_t)li] |= 1 | 2;
+    return GAO_OK;
+}
+
+// The program's stream waits for a pass's copies back on the third stream, if any are queued
+// (a captured graph needs them joined too).
+gao_status join_outputs(RunCtx& R) {
+    if (!R.out_pending) return GAO_OK;
+    R.out_pending = false;
+    GAO_CUDA_TRY(cudaStreamWaitEvent(R.st, R.p->out_ev[(size_t)kMaxRowBlocks], 0));
     return GAO_OK;
 }
 
@@ -1615,11 +1677,17 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
             // the image comes from the host: strips overlapped with its copy, with the
             // gradient chain on this stencil's output in the same strips when the gene fuses it
             const bool chained = find_edge_chain(p, li, gene_mask, fuse, &gch);
-            if ((status = run_gpu_stencil_pipelined(R, li, chained ? &gch : nullptr)) != GAO_OK) break;
+            std::vector<int> on_host;
+            const int after = chained ? std::max({li + 5, gch.sum_loop, gch.colmax_loop}) + 1 : li + 1;
+            if ((status = join_outputs(R)) != GAO_OK) break;
+            if ((status = run_gpu_stencil_pipelined(R, li, chained ? &gch : nullptr, !(flags & GAO_RUN_KEEP_DEVICE),
+                                                    after, &on_host)) != GAO_OK)
+                break;
             BufState& Bo = p->bufs[(size_t)L.outs[0]];
             Bo.vh = false;
             Bo.vd = true;
             if (chained) grad_chain_done(p, gch, li + 1, &fused);
+            for (int b : on_host) p->bufs[(size_t)b].vh = true;  // copied back strip by strip
             if (R.deadline > 0.0 && now_s() > R.deadline) R.timed_out = true;
             if (R.timed_out) break;
             continue;
@@ -1812,6 +1880,7 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
             const bool early_out = !per_loop && !(flags & GAO_RUN_KEEP_DEVICE) && Cb.d.role == GAO_BUF_OUTPUT &&
                                    Cb.host != nullptr && L.outs[0] != L.ins[0] && L.outs[0] != L.ins[1];
             c_on_host = false;
+            if ((status = join_outputs(R)) != GAO_OK) break;
             if ((status = run_gpu_gemm_pipelined(R, li, blocks, pf ? &pch : nullptr, early_out, &c_on_host)) !=
                 GAO_OK)
                 break;
@@ -1852,6 +1921,7 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
             if (status != GAO_OK) break;
             // the host loop may overwrite mirrors that queued copies still read, and
             // reads mirrors that queued copies fill: drain the stream first
+            if ((status = join_outputs(R)) != GAO_OK) break;
             if (uses_gpu && (status = stream_wait(p->st, R.deadline, &R.timed_out)) != GAO_OK) break;
             const double c1 = now_s();
             S.copy_ms = (c1 - c0) * 1e3;
@@ -1883,6 +1953,8 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
         if (!p->stats.empty()) p->stats.back().d2h_bytes += dummy.d2h_bytes;
     }
     if (uses_gpu) {
+        const gao_status js = join_outputs(R);
+        if (js != GAO_OK && status == GAO_OK) status = js;
         cudaError_t e = cudaMemcpyAsync(p->h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, p->st);
         if (e != cudaSuccess && status == GAO_OK) status = cuda_fail(e, "cudaMemcpyAsync(err)");
     }
