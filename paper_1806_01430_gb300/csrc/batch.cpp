@@ -586,21 +586,23 @@ gao_status run_genes(gao_batch* b, const uint64_t* genes, int u, double* seconds
         }
         if (!attributed && budget > 0.0 && now_s() - t0 > budget) dead[0] = 1;
     }
+    HostCopySet small;
+    small.n = 0;
+    gao_status s = GAO_OK;
     for (int r = 0; r < u; ++r) {
         if (dead[(size_t)r]) continue;
         GAO_CUDA_TRY(rec(eout(r, 0)));
         for (auto& c : rc[(size_t)r])
             for (size_t bi = 0; bi < c.p->bufs.size(); ++bi)
-                if (c.p->bufs[bi].d.role == GAO_BUF_OUTPUT && !c.p->bufs[bi].vh) {
-                    gao_status s = make_valid(c, (int)bi, false, scratch);
-                    if (s != GAO_OK) return s;
-                }
+                if (c.p->bufs[bi].d.role == GAO_BUF_OUTPUT && !c.p->bufs[bi].vh)
+                    if ((s = output_to_host(c, (int)bi, small, scratch)) != GAO_OK) return s;
+        if ((s = send_small(small, b->st)) != GAO_OK) return s;
         GAO_CUDA_TRY(rec(eout(r, 1)));
         if (attributed) out_used[(size_t)r] = 1;
     }
-    GAO_CUDA_TRY(cudaMemcpyAsync(b->h_err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->st));
+    if ((s = send_small(small, b->st, b->d_err, b->h_err)) != GAO_OK) return s;
     bool to = false;
-    gao_status s = stream_wait(b->st, 0.0, &to);
+    s = stream_wait(b->st, 0.0, &to);
     if (s != GAO_OK) return s;
     const double t1 = now_s();
     spans_ready = attributed && launched;

@@ -114,6 +114,19 @@ struct InitEntry {
     int64_t start4;
 };
 cudaError_t launch_init_group(const InitEntry* d_tab, int n_entries, int64_t total4, cudaStream_t st);
+// Small outputs to their page-locked host mirrors (16-byte aligned, like the device buffers).
+struct HostCopy {
+    const void* src;
+    void* dst;
+    uint32_t words;  // of 4 bytes
+};
+constexpr int kMaxHostCopies = 128;
+constexpr size_t kHostCopyBytes = 512u << 10;  // largest buffer copied this way
+struct HostCopySet {
+    int n;
+    HostCopy c[kMaxHostCopies];
+};
+cudaError_t launch_host_copies(const HostCopySet& set, cudaStream_t st);
 cudaError_t launch_axpy(float* out, const float* x, float alpha, const float* y, int64_t n, cudaStream_t st);
 cudaError_t launch_transpose(float* out, const float* in, int64_t rows, int64_t cols, cudaStream_t st);
 // Row sums (ROWSUM) follow one fixed order on every path -- the row-sum kernel, the fused

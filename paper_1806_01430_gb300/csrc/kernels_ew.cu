@@ -219,6 +219,22 @@ __global__ void ew_kernel(float* __restrict__ out, const float* __restrict__ x, 
         out[i] = ew_apply<OP>(x[i], OP == Ew::Axpy ? y[i] : 0.0f, alpha);
 }
 
+// ---- small outputs to the host ------------------------------------------------------------
+//
+// One launch stores a run's small outputs (and its error word) into their page-locked mirrors
+// over the link.  A copy of its own costs each output a transfer's start, which they pay one
+// after the other on the run's stream (a batch's gene over 16 programs of three outputs: 775 -> 733
+// us; a six-loop step at 256: 117 -> 111); above kHostCopyBytes a transfer's start is lost
+// in its time on the link, and the copy engine needs no SM.
+__global__ void __launch_bounds__(kThreads) host_copies_kernel(const __grid_constant__ HostCopySet set) {
+    const HostCopy& c = set.c[blockIdx.y];
+    const uint32_t quads = c.words / 4, stride = gridDim.x * kThreads, t = blockIdx.x * kThreads + threadIdx.x;
+    for (uint32_t i = t; i < quads; i += stride)
+        reinterpret_cast<uint4*>(c.dst)[i] = reinterpret_cast<const uint4*>(c.src)[i];
+    const uint32_t w = quads * 4 + t;
+    if (w < c.words) reinterpret_cast<uint32_t*>(c.dst)[w] = reinterpret_cast<const uint32_t*>(c.src)[w];
+}
+
 // ---- element-wise chains ---------------------------------------------------------------
 
 // Consecutive element-wise loops (RELU, SQUARE, AXPY) over the same shape in one pass.
@@ -1389,6 +1405,16 @@ cudaError_t launch_ew_chain(const EwChain& c, cudaStream_t st) {
     k.vec = chain_fields(k);
     if (k.next > 0) ew_chain_kernel<true><<<grid_for((c.n + 7) / 8), kThreads, 0, st>>>(k);
     else ew_chain_kernel<false><<<grid_for((c.n + 3) / 4), kThreads, 0, st>>>(k);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_host_copies(const HostCopySet& set, cudaStream_t st) {
+    if (set.n < 1) return cudaSuccess;
+    if (set.n > kMaxHostCopies) return cudaErrorInvalidValue;
+    uint32_t words = 0;
+    for (int k = 0; k < set.n; ++k) words = std::max(words, set.c[k].words);
+    const dim3 grid(std::min<uint32_t>(32, words / 4 / kThreads + 1), (unsigned)set.n);
+    host_copies_kernel<<<grid, kThreads, 0, st>>>(set);
     return cudaGetLastError();
 }
 

@@ -609,6 +609,38 @@ gao_status make_valid(RunCtx& R, int b, bool on_gpu, gao_loop_stat& stat) {
     return GAO_OK;
 }
 
+gao_status send_small(HostCopySet& set, cudaStream_t st, const int* d_err, int* h_err) {
+    if (d_err) {
+        if (set.n == 0) {
+            GAO_CUDA_TRY(cudaMemcpyAsync(h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+            return GAO_OK;
+        }
+        if (set.n == kMaxHostCopies) {
+            GAO_CUDA_TRY(launch_host_copies(set, st));
+            set.n = 0;
+        }
+        set.c[set.n++] = HostCopy{d_err, h_err, 1};
+    }
+    GAO_CUDA_TRY(launch_host_copies(set, st));
+    set.n = 0;
+    return GAO_OK;
+}
+
+gao_status output_to_host(RunCtx& R, int b, HostCopySet& set, gao_loop_stat& stat) {
+    BufState& B = R.p->bufs[(size_t)b];
+    if (B.vh) return GAO_OK;
+    if (!B.vd || B.host != B.own_host || B.bytes == 0 || B.bytes > kHostCopyBytes || B.bytes % 4 != 0)
+        return make_valid(R, b, false, stat);
+    if (set.n == kMaxHostCopies) {
+        const gao_status s = send_small(set, R.st);
+        if (s != GAO_OK) return s;
+    }
+    set.c[set.n++] = HostCopy{B.dev, B.host, (uint32_t)(B.bytes / 4)};
+    stat.d2h_bytes += B.bytes;
+    B.vh = true;
+    return GAO_OK;
+}
+
 std::vector<int> loop_inputs(const gao_loop& L) {
     std::vector<int> v;
     if (L.kind == GAO_LOOP_INIT) return v;
@@ -1945,18 +1977,20 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
         if (R.deadline > 0.0 && now_s() > R.deadline) R.timed_out = true;
         if (R.timed_out) break;
     }
+    HostCopySet small;
+    small.n = 0;
     if (status == GAO_OK && !R.timed_out && !(flags & GAO_RUN_KEEP_DEVICE)) {
         gao_loop_stat dummy{};
         for (size_t b = 0; b < p->bufs.size(); ++b)
             if (p->bufs[b].d.role == GAO_BUF_OUTPUT && !p->bufs[b].vh)
-                if ((status = make_valid(R, (int)b, false, dummy)) != GAO_OK) break;
+                if ((status = output_to_host(R, (int)b, small, dummy)) != GAO_OK) break;
         if (!p->stats.empty()) p->stats.back().d2h_bytes += dummy.d2h_bytes;
     }
     if (uses_gpu) {
-        const gao_status js = join_outputs(R);
-        if (js != GAO_OK && status == GAO_OK) status = js;
-        cudaError_t e = cudaMemcpyAsync(p->h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, p->st);
-        if (e != cudaSuccess && status == GAO_OK) status = cuda_fail(e, "cudaMemcpyAsync(err)");
+        gao_status es = join_outputs(R);
+        if (es != GAO_OK && status == GAO_OK) status = es;
+        es = send_small(small, p->st, (const int*)d_err, p->h_err);
+        if (es != GAO_OK && status == GAO_OK) status = es;
     }
     return status;
 }
