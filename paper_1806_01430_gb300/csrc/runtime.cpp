@@ -1602,15 +1602,17 @@ double ev_ms(cudaEvent_t a, cudaEvent_t b) {
 // (*which = 1), when that GEMM runs on the GPU in split bfloat16 without a fused chain: b is
 // then formed straight into the GEMM's bfloat16 planes, never as binary32.  -1 otherwise (b
 // is not a TEMP buffer, is read by anything else or written by another loop, the GEMM reads
-// it twice or also as C0, transfers are per loop).
+// it twice or also as C0, another GEMM on the GPU uses the one room for planes, transfers are
+// per loop).
 int planes_consumer(const gao_prog* p, int li, int b, uint64_t gene_mask, bool fuse, int* which) {
     const BufState& B = p->bufs[(size_t)b];
     if (B.d.role != GAO_BUF_TEMP || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT || p->lay.tc_bytes == 0) return -1;
     const int prec = p->opts.gemm_prec;
     if (prec != GAO_GEMM_BF16 && prec != GAO_GEMM_BF16X3 && prec != GAO_GEMM_BF16X6) return -1;
-    int reader = -1;
+    int reader = -1, gemms = 0;
     for (int j = 0; j < (int)p->loops.size(); ++j) {
         const gao_loop& Lj = p->loops[(size_t)j];
+        if (Lj.kind == GAO_LOOP_GEMM && ((gene_mask >> j) & 1) && ++gemms > 1) return -1;
         if (j != li)
             for (int o : loop_outputs(Lj))
                 if (o == b) return -1;
