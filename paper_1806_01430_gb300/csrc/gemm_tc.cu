@@ -1724,12 +1724,12 @@ TcShape tc_shape(int prec, int64_t M, int64_t Mlay, int64_t N, int64_t K, int kc
 }  // namespace
 
 cudaError_t tc_init_planes(int prec, int which, int64_t M, int64_t N, int64_t K, int kchunk, int tile_cfg,
-                           uint64_t seed, uint32_t buf, const int8_t* rowexp, void* scratch, size_t scratch_bytes,
+                           bool chain, uint64_t seed, uint32_t buf, const int8_t* rowexp, void* scratch, size_t scratch_bytes,
                            cudaStream_t st, int* launches) {
     *launches = 0;
     if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_BF16X6 || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
     if (tc_scratch_bytes(prec, M, N, K) > scratch_bytes || ((uintptr_t)scratch & 1023u)) return cudaErrorInvalidValue;
-    const TcShape g = tc_shape(prec, M, M, N, K, kchunk, tile_cfg, nullptr, false);
+    const TcShape g = tc_shape(prec, M, M, N, K, kchunk, tile_cfg, nullptr, chain);
     __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(scratch);
     if (which == 0) {  // A (M x K) -> [P][Mp][Kp]
         int64_t blocks = (g.Mp * (g.Kp / 8) + 255) / 256;

@@ -90,6 +90,7 @@ namespace gao {
 constexpr int kMaxRowBlocks = 4;                 // row blocks of an overlapped GEMM loop
 constexpr int kMaxColParts = 2;                  // column ranges of its first row block
 constexpr size_t kPipelineMinBytes = 16u << 20;  // smallest A worth overlapping
+constexpr size_t kPlanesMinBytes = 16u << 20;    // smallest operand of a GEMM with its chain formed as planes
 
 // One execution of a program (or of a batch of programs sharing a stream).
 struct RunCtx {

@@ -660,6 +660,12 @@ std::vector<int> loop_outputs(const gao_loop& L) {
     return v;
 }
 
+// GEMM loop li's operands that an INIT loop formed straight into its planes (bit 0: A, bit 1: B).
+unsigned planes_ready(const gao_prog* p, int li) {
+    const gao_loop& G = p->loops[(size_t)li];
+    return (p->bufs[(size_t)G.ins[0]].gen_for == li ? 1u : 0u) | (p->bufs[(size_t)G.ins[1]].gen_for == li ? 2u : 0u);
+}
+
 gao_status run_gpu_loop(RunCtx& R, int li) {
     gao_prog* p = R.p;
     const gao_loop& L = p->loops[(size_t)li];
@@ -713,13 +719,10 @@ gao_status run_gpu_loop(RunCtx& R, int li) {
             } else {
                 std::string why;
                 TcEvents tev{k0, k1, 0};
-                // operands an INIT loop formed straight into this GEMM's planes
-                const unsigned ready = (p->bufs[(size_t)L.ins[0]].gen_for == li ? 1u : 0u) |
-                                       (p->bufs[(size_t)L.ins[1]].gen_for == li ? 2u : 0u);
                 e = launch_gemm_tc(prec, dptr(L.outs[0]), dptr(L.ins[0]), dptr(L.ins[1]), c0 ? c0 : dptr(L.outs[0]),
                                    A.rows, B.cols, A.cols, (float)L.alpha, beta, p->opts.kchunk, p->opts.tile_cfg,
                                    a + p->lay.tc_off, p->lay.tc_bytes, d_err, st, tev, &why, nullptr, nullptr,
-                                   ready);
+                                   planes_ready(p, li));
                 if (e != cudaSuccess && !why.empty()) return fail(GAO_EINVAL, "tensor-core GEMM: " + why);
                 nl += tev.launches;
             }
@@ -1219,7 +1222,8 @@ gao_status run_gpu_chain(RunCtx& R, int li, const Chain& ch) {
     cudaError_t e = launch_gemm_tc(p->opts.gemm_prec, dptr(G.outs[0]), dptr(G.ins[0]), dptr(G.ins[1]), c0, A.rows,
                                    B.cols, A.cols, (float)G.alpha, G.ins[2] >= 0 ? (float)G.beta : 0.0f,
                                    p->opts.kchunk, p->opts.tile_cfg, p->arena + p->lay.tc_off, p->lay.tc_bytes,
-                                   (int*)(p->arena + p->lay.err_off), R.st, tev, &why, &fz);
+                                   (int*)(p->arena + p->lay.err_off), R.st, tev, &why, &fz, nullptr,
+                                   planes_ready(p, li));
     if (e != cudaSuccess) return why.empty() ? cuda_fail(e, "fused chain launch") : fail(GAO_EINVAL, why);
     p->stats[(size_t)li].launches += tev.launches;
     p->ev_used[(size_t)li] |= 4;
@@ -1599,11 +1603,13 @@ double ev_ms(cudaEvent_t a, cudaEvent_t b) {
 // kernels (or its host loop), the outputs' copies back and the error word's read-back.
 // When every loop is on the GPU this is also what a CUDA graph of the run captures.
 // The GEMM loop that alone reads INIT loop li's output b, as its A (*which = 0) or its B
-// (*which = 1), when that GEMM runs on the GPU in split bfloat16 without a fused chain: b is
-// then formed straight into the GEMM's bfloat16 planes, never as binary32.  -1 otherwise (b
-// is not a TEMP buffer, is read by anything else or written by another loop, the GEMM reads
-// it twice or also as C0, another GEMM on the GPU uses the one room for planes, transfers are
-// per loop).
+// (*which = 1), when that GEMM runs on the GPU in split bfloat16: b is then formed straight
+// into the GEMM's bfloat16 planes, never as binary32.  A GEMM with its chain takes operands of
+// at least kPlanesMinBytes this way; below that the split it saves is a few us.  Whole pass:
+// six-loop program 4096, three terms, B: 664 -> 643 us; twelve-loop 6000, K = 1500, two terms, A
+// and B: 455 -> 435.  -1 otherwise (b is not a TEMP buffer, is read by anything else or written
+// by another loop, the GEMM reads it twice or also as C0, another GEMM on the GPU uses the one
+// room for planes, transfers are per loop).
 int planes_consumer(const gao_prog* p, int li, int b, uint64_t gene_mask, bool fuse, int* which) {
     const BufState& B = p->bufs[(size_t)b];
     if (B.d.role != GAO_BUF_TEMP || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT || p->lay.tc_bytes == 0) return -1;
@@ -1627,7 +1633,12 @@ int planes_consumer(const gao_prog* p, int li, int b, uint64_t gene_mask, bool f
     if (G.kind != GAO_LOOP_GEMM || !((gene_mask >> reader) & 1)) return -1;
     if (G.outs[0] == b || G.ins[2] == b || (G.ins[0] == b) == (G.ins[1] == b)) return -1;
     Chain c;
-    if (find_chain(p, reader, gene_mask, fuse, &c)) return -1;
+    if (find_chain(p, reader, gene_mask, fuse, &c)) {
+        // A still to come from the host would run in row blocks, which split their operands
+        const std::vector<int> mine = loop_outputs(p->loops[(size_t)li]);
+        const bool a_here = p->bufs[(size_t)G.ins[0]].vd || std::find(mine.begin(), mine.end(), G.ins[0]) != mine.end();
+        if (B.bytes < kPlanesMinBytes || !a_here) return -1;
+    }
     const gao_buffer &A = p->bufs[(size_t)G.ins[0]].d, &Bm = p->bufs[(size_t)G.ins[1]].d;
     if (A.rows <= 0 || A.cols <= 0 || Bm.cols <= 0) return -1;
     *which = G.ins[0] == b ? 0 : 1;
@@ -1670,8 +1681,9 @@ gao_status run_gpu_init_planes(RunCtx& R, int li, const int* cons, const int* wh
         const gao_buffer &A = p->bufs[(size_t)G.ins[0]].d, &Bm = p->bufs[(size_t)G.ins[1]].d;
         const int rs = (int)((L.flags >> t) & 1);
         int l = 0;
+        Chain ch;
         GAO_CUDA_TRY(tc_init_planes(p->opts.gemm_prec, wh[t], A.rows, Bm.cols, A.cols, p->opts.kchunk,
-                                    p->opts.tile_cfg, p->opts.seed, (uint32_t)L.outs[t], rs ? set.rowexp : nullptr,
+                                    p->opts.tile_cfg, find_chain(p, cons[t], p->run_mask, p->run_fuse, &ch), p->opts.seed, (uint32_t)L.outs[t], rs ? set.rowexp : nullptr,
                                     a + p->lay.tc_off, p->lay.tc_bytes, st, &l));
         nl += l;
     }
@@ -1870,6 +1882,8 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
             std::vector<int> cin = loop_inputs(L);
             cin.push_back(p->loops[(size_t)chain.axpy].ins[1]);
             bool copies = false;
+            cin.erase(std::remove_if(cin.begin(), cin.end(), [&](int b) { return p->bufs[(size_t)b].gen_for == li; }),
+                      cin.end());  // read as planes
             for (int b : cin) copies |= !p->bufs[(size_t)b].vd;
             if (copies) GAO_CUDA_TRY(record_timing(ev[0], p->st));
             for (int b : cin)

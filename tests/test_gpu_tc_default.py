@@ -18,9 +18,10 @@ def gao():
     return g
 
 
-def chain_program(m, k, n):
+def chain_program(m, k, n, keep):
     o = W.OUTPUT
-    bufs = [W.Buffer("A", m, k), W.Buffer("B", k, n), W.Buffer("C", m, n, role=o), W.Buffer("S", m, n),
+    ab = o if keep else W.TEMP  # kept: split by the GEMM; else formed as planes where large enough
+    bufs = [W.Buffer("A", m, k, role=ab), W.Buffer("B", k, n, role=ab), W.Buffer("C", m, n, role=o), W.Buffer("S", m, n),
             W.Buffer("D", m, n), W.Buffer("E", n, m, role=o), W.Buffer("r", n, 1, role=o),
             W.Buffer("f", 1, 1, W.F64, o)]
     L = W.Loop
@@ -32,13 +33,15 @@ def chain_program(m, k, n):
 @pytest.mark.parametrize("m,k,n", [(3968, 1500, 3840), (3968, 1499, 3840), (3841, 1600, 3969), (3840, 1500, 3712),
                                    (2433, 1500, 3072)])
 def test_chain_default_against_one_cta(gao, prec, m, k, n):
-    bufs, loops = chain_program(m, k, n)
     got = []
-    for cfg in (0, 1, 9):
+    for cfg, keep in ((0, False), (0, True), (1, False), (9, True), (13, False)):
+        bufs, loops = chain_program(m, k, n, keep)
         p = gao.prog_create(bufs, loops, seed=3, gemm_prec=PREC[prec], tile_cfg=cfg, fuse_chains=1)
         gao.prog_run(p, 0b111111)
         got.append([gao.prog_output(p, b).copy() for b in (2, 5, 6, 7)])
-        assert gao.prog_stats(p)[1]["launches"] == 5
+        planes = [not keep and 4 * x >= 1 << 24 for x in (m * k, k * n)]
+        assert [gao.prog_planes_for(p, b) == 1 for b in (0, 1)] == planes
+        assert gao.prog_stats(p)[1]["launches"] == 5 - sum(planes)
         gao.prog_destroy(p)
     for g in got[1:]:
         for a, b in zip(got[0][:3], g[:3]):
