@@ -411,8 +411,9 @@ def group_bytes(prog, idx, planes=None) -> float:
 
 
 def planes_of_run(gao, p, prog, prec):
-    """Buffers the last run formed only as a GEMM's bfloat16 planes -> planes per element."""
-    P = {"bf16": 1, "bf16x3": 2, "bf16x6": 3}.get(prec)
+    """Buffers the last run formed only as a GEMM's bfloat16 planes -> planes per element (FP8's
+    one byte an element counts as half a plane)."""
+    P = {"bf16": 1, "bf16x3": 2, "bf16x6": 3, "fp8": 0.5}.get(prec)
     if P is None:
         return {}
     return {b: P for b in range(len(prog.buffers)) if gao.prog_planes_for(p, b) >= 0}

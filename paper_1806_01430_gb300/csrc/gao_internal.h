@@ -288,7 +288,7 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
                            int64_t N, int64_t K, float alpha, float beta, int kchunk, int tile_cfg, void* scratch,
                            size_t scratch_bytes, int* err, cudaStream_t st, TcEvents& ev, std::string* why,
                            const TcFuse* fuse = nullptr, const TcPart* part = nullptr, unsigned ready = 0);
-// The bfloat16 planes of operand `which` (0: A, M x K; 1: B, K x N) of that GEMM (same
+// The bfloat16 planes (FP8: e4m3 codes and scales) of operand `which` (0: A, M x K; 1: B, K x N) of that GEMM (same
 // precision, shapes, K chunk and tile configuration; chain: with `fuse`), formed in its scratch straight from the
 // INIT loop's counter hash of buffer `buf` (times 2^e of each row where rowexp is set), with
 // the values, splitting and zero padding of INIT followed by the GEMM's own split.

@@ -1373,11 +1373,37 @@ __device__ __forceinline__ void put_sf(uint8_t* blk, int r, int e) {
     *reinterpret_cast<uint32_t*>(blk + 16 * (r & 31) + 4 * (r >> 5)) = (uint32_t)(e + 127) * 0x01010101u;
 }
 
+// An operand that an INIT loop forms and nothing but this GEMM reads: its element idx is
+// init_value(seed, buf, idx), times 2^e of its row where rowexp is set.  The quantise kernels
+// then form the elements where they would load them (GEN), and the binary32 array, which cost
+// a write and a read of four bytes an element, is never written (3000 x 5003 x 4100, both
+// operands, INIT and quantisation: 74 -> 68 us).
+struct InitSrc {
+    uint64_t seed;
+    uint32_t buf;
+    const int8_t* rowexp;
+};
+// Elements idx0 .. idx0 + N - 1 (N even) from the hashes of idx0 / 2 .. (idx0 + N - 1) / 2.
+template <int N>
+__device__ __forceinline__ void init_gen(const InitSrc& g, uint64_t idx0, float (&x)[N]) {
+    const bool odd = (idx0 & 1) != 0;
+    uint64_t h[N / 2 + 1];
+#pragma unroll
+    for (int j = 0; j <= N / 2; ++j) h[j] = (j < N / 2 || odd) ? sm64_hash(init_key(g.seed, g.buf, (idx0 >> 1) + j)) : 0;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {  // the high 24 bits of hash idx / 2 for an even idx, bits 16..39 for an odd one
+        const uint64_t e = (q & 1) ? h[q / 2] >> 16 : h[q / 2] >> 40;
+        const uint64_t o = (q & 1) ? h[q / 2 + 1] >> 40 : h[q / 2] >> 16;
+        x[q] = u24_to_value((uint32_t)((odd ? o : e) & 0xFFFFFFu));
+    }
+}
+
 // A (M x K) -> q [Mp][Kp] e4m3 and scale-factor blocks sfa [Mp / 128][Kp / 128][512 bytes];
 // one warp per (row, K block), lane = 4 k, kQuantAhead blocks' loads in flight.  HBM-bound (5
 // bytes an element): 3000 x 4100 in 21.5 us, 24.2 with one block's loads at a time.
 constexpr int kQuantAhead = 4;
-__global__ void __launch_bounds__(256) quant_rows_fp8_kernel(const float* __restrict__ A, int64_t M, int64_t K,
+template <bool GEN>
+__global__ void __launch_bounds__(256) quant_rows_fp8_kernel(const float* __restrict__ A, InitSrc gen, int64_t M, int64_t K,
                                                              int64_t Mp, int64_t Kp, uint8_t* __restrict__ q,
                                                              uint8_t* __restrict__ sfa) {
     const int lane = threadIdx.x & 31;
@@ -1385,17 +1411,33 @@ __global__ void __launch_bounds__(256) quant_rows_fp8_kernel(const float* __rest
     const int64_t nwork = Mp * kbs;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const bool vec = (K % 4 == 0) && (((uintptr_t)A & 15u) == 0);
-    for (int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; w0 < nwork; w0 += kQuantAhead * nwarps) {
+    // (row, K block) advanced by the stride's quotient and remainder: no 64-bit division in the loop
+    int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t di = nwarps / kbs, dk = nwarps % kbs;
+    int64_t next_row = w0 / kbs, next_kb = w0 % kbs;
+    for (; w0 < nwork; w0 += kQuantAhead * nwarps) {
         float x[kQuantAhead][4];
         int64_t row[kQuantAhead], kb[kQuantAhead];
 #pragma unroll
         for (int u = 0; u < kQuantAhead; ++u) {
             const int64_t w = w0 + u * nwarps;
-            row[u] = w / kbs;
-            kb[u] = w - row[u] * kbs;
+            row[u] = next_row;
+            kb[u] = next_kb;
+            next_row += di;
+            next_kb += dk;
+            if (next_kb >= kbs) {
+                next_kb -= kbs;
+                ++next_row;
+            }
             const int64_t k0 = kb[u] * 128 + lane * 4;
             const bool in = w < nwork && row[u] < M;
-            if (vec) {  // four elements are wholly inside or outside the row
+            if constexpr (GEN) {
+                float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                if (in && k0 < K) init_gen(gen, (uint64_t)(row[u] * K + k0), v);
+                const int e = gen.rowexp && in ? gen.rowexp[row[u]] : 0;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) x[u][t] = k0 + t < K ? (gen.rowexp ? ldexpf(v[t], e) : v[t]) : 0.0f;
+            } else if (vec) {  // four elements are wholly inside or outside the row
                 float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 if (in && k0 < K) v = __ldg(reinterpret_cast<const float4*>(A + row[u] * K + k0));
                 x[u][0] = v.x, x[u][1] = v.y, x[u][2] = v.z, x[u][3] = v.w;
@@ -1425,31 +1467,77 @@ __global__ void __launch_bounds__(256) quant_rows_fp8_kernel(const float* __rest
 // whole 128-byte rows of q^T.  HBM-bound: 4100 x 5003 in 20.7 us = 5.0 TB/s; 48.1
 // with a row's load waited for at a time and a column's packing lanes in conflict on its banks.
 constexpr int kQuantCols = 64;
-__global__ void __launch_bounds__(256) quant_cols_fp8_kernel(const float* __restrict__ B, int64_t K, int64_t N,
+template <bool GEN>
+__global__ void __launch_bounds__(256) quant_cols_fp8_kernel(const float* __restrict__ B, InitSrc gen, int64_t K, int64_t N,
                                                              int64_t Np, int64_t Kp, uint8_t* __restrict__ q,
                                                              uint8_t* __restrict__ sfb) {
     __shared__ __align__(16) float tile[128][kQuantCols + 1];
-    __shared__ float red[4][kQuantCols];
+    constexpr int kRed = GEN ? 8 : 4;
+    __shared__ float red[kRed][kQuantCols];
     __shared__ float scale[kQuantCols];
     const int t = threadIdx.x, c = t & (kQuantCols - 1), g = t / kQuantCols;  // column; row group
     const int64_t kb = blockIdx.y, n0 = (int64_t)blockIdx.x * kQuantCols;
     const int64_t kbs = Kp / 128;
-    const float* src = B + (kb * 128 + g) * N + n0 + c;
-    const bool cin = n0 + c < N;
     const int rows = (int)(K - kb * 128 < 128 ? K - kb * 128 : 128);  // of this K block inside K
-    float v[32];
+    if constexpr (GEN) {
+        // A warp takes every eighth row, a lane the two columns that share a hash: c2 and c2 + 1,
+        // or, where the row's elements start at an odd index (an odd N, an odd row), c2 - 1 and
+        // c2, which leaves the last column of such rows to a pass of its own, a row per lane.
+        const int lane = t & 31, g8 = t >> 5, odd = (int)(N & 1) & g8;
+        const int ca = 2 * lane - odd, cb = ca + 1;
+        const bool in_a = ca >= 0 && n0 + ca < N, in_b = n0 + cb < N;
+        float ma = 0.0f, mb = 0.0f;
+#pragma unroll 4
+        for (int r = g8; r < 128; r += 8) {
+            float va = 0.0f, vb = 0.0f;
+            if (r < rows && (in_a || in_b)) {
+                const int64_t k = kb * 128 + r;
+                const uint64_t h = sm64_hash(init_key(gen.seed, gen.buf, (uint64_t)(k * N + n0 + cb) >> 1));
+                if (in_a) va = u24_to_value((uint32_t)(h >> 40));
+                if (in_b) vb = u24_to_value((uint32_t)((h >> 16) & 0xFFFFFFu));
+                if (gen.rowexp) {
+                    va = ldexpf(va, gen.rowexp[k]);
+                    vb = ldexpf(vb, gen.rowexp[k]);
+                }
+            }
+            if (ca >= 0) tile[r][ca] = va;
+            tile[r][cb] = vb;
+            ma = fmaxf(ma, fabsf(va));
+            mb = fmaxf(mb, fabsf(vb));
+        }
+        if (ca >= 0) red[g8][ca] = ma;
+        red[g8][cb] = mb;
+        if (odd) {
+            const int r = g8 + 8 * (lane & 15);
+            const int64_t k = kb * 128 + r;
+            float v = r < rows && n0 + kQuantCols - 1 < N
+                          ? init_value(gen.seed, gen.buf, (uint64_t)(k * N + n0 + kQuantCols - 1)) : 0.0f;
+            if (gen.rowexp && r < rows) v = ldexpf(v, gen.rowexp[k]);
+            tile[r][kQuantCols - 1] = v;
+            v = fabsf(v);
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = (cin && g + 4 * i < rows) ? __ldg(src + (int64_t)(4 * i) * N) : 0.0f;
-    float m = 0.0f;
+            for (int off = 8; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+            if (lane == 0) red[g8][kQuantCols - 1] = v;
+        }
+    } else {
+        const float* src = B + (kb * 128 + g) * N + n0 + c;
+        const bool cin = n0 + c < N;
+        float v[32];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        tile[g + 4 * i][c] = v[i];
-        m = fmaxf(m, fabsf(v[i]));
+        for (int i = 0; i < 32; ++i) v[i] = (cin && g + 4 * i < rows) ? __ldg(src + (int64_t)(4 * i) * N) : 0.0f;
+        float m = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            tile[g + 4 * i][c] = v[i];
+            m = fmaxf(m, fabsf(v[i]));
+        }
+        red[g][c] = m;
     }
-    red[g][c] = m;
     __syncthreads();
     if (t < kQuantCols) {
-        const float a = fmaxf(fmaxf(red[0][t], red[1][t]), fmaxf(red[2][t], red[3][t]));
+        float a = red[0][t];
+#pragma unroll
+        for (int j = 1; j < kRed; ++j) a = fmaxf(a, red[j][t]);
         const int e = fp8_block_exp(a);
         scale[t] = fp8_scale(e);
         const int64_t n = n0 + t;
@@ -1600,7 +1688,7 @@ cudaError_t launch_mma_pair(const CUtensorMap& ta, const CUtensorMap& tb, const 
 
 cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N, int64_t K,
                             float alpha, float beta, int tile_cfg, void* scratch, size_t scratch_bytes, int* err,
-                            cudaStream_t st, TcEvents& ev, std::string* why);
+                            cudaStream_t st, TcEvents& ev, std::string* why, unsigned ready);
 
 // Epilogue warps of a launch.  An epilogue bound by the latency of its C0 / X loads and staging
 // round trips takes sixteen: rows that are not 16-byte aligned, a word a lane (GEMM with
@@ -1636,6 +1724,26 @@ Fp8Layout fp8_layout(int64_t M, int64_t N, int64_t K) {
     L.total = L.sb + ru((L.Np / 128) * L.kbs * kSfBlock, 1024);
     return L;
 }
+
+namespace {
+// Operand `which` of the FP8 GEMM quantised (from X, or from the INIT loop's hash) at its place
+// in the scratch.
+template <bool GEN>
+cudaError_t quant_fp8(int which, const float* X, const InitSrc& gen, int64_t M, int64_t N, int64_t K, uint8_t* base,
+                      cudaStream_t st) {
+    const Fp8Layout L = fp8_layout(M, N, K);
+    if (which == 0) {
+        const int64_t warps = L.Mp * L.kbs;
+        const int64_t g = std::min<int64_t>((warps * 32 + 255) / 256, (int64_t)sm_count() * 8);
+        quant_rows_fp8_kernel<GEN><<<(unsigned)g, 256, 0, st>>>(X, gen, M, K, L.Mp, L.Kp, base + L.qa, base + L.sa);
+    } else {
+        const dim3 grid((unsigned)(L.Np / kQuantCols), (unsigned)L.kbs);
+        if (grid.y > 65535u) return cudaErrorInvalidValue;
+        quant_cols_fp8_kernel<GEN><<<grid, 256, 0, st>>>(X, gen, K, N, L.Np, L.Kp, base + L.qb, base + L.sb);
+    }
+    return cudaGetLastError();
+}
+}  // namespace
 
 // Planes (or FP8 arrays) first, then binary64 partials for a fused chain's norm
 // (16 per 128 x 128 tile), then its row sums' 32-row block values (binary32, [Mp / 32][N]).
@@ -1727,8 +1835,12 @@ cudaError_t tc_init_planes(int prec, int which, int64_t M, int64_t N, int64_t K,
                            bool chain, uint64_t seed, uint32_t buf, const int8_t* rowexp, void* scratch, size_t scratch_bytes,
                            cudaStream_t st, int* launches) {
     *launches = 0;
-    if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_BF16X6 || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
+    if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_FP8 || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
     if (tc_scratch_bytes(prec, M, N, K) > scratch_bytes || ((uintptr_t)scratch & 1023u)) return cudaErrorInvalidValue;
+    if (prec == GAO_GEMM_FP8) {
+        *launches = 1;
+        return quant_fp8<true>(which, nullptr, InitSrc{seed, buf, rowexp}, M, N, K, static_cast<uint8_t*>(scratch), st);
+    }
     const TcShape g = tc_shape(prec, M, M, N, K, kchunk, tile_cfg, nullptr, chain);
     __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(scratch);
     if (which == 0) {  // A (M x K) -> [P][Mp][Kp]
@@ -1781,7 +1893,7 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
             return cudaErrorInvalidValue;
         }
         return launch_gemm_fp8(C, A, B, C0, M, N, K, alpha, beta, tile_cfg, scratch, scratch_bytes, err, st, ev,
-                               why);
+                               why, ready);
     }
     const int64_t Mlay = part ? part->m_layout : M;
     if (Mlay < M || (part && ready)) {
@@ -1912,7 +2024,7 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
 namespace {
 cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N, int64_t K,
                             float alpha, float beta, int tile_cfg, void* scratch, size_t scratch_bytes, int* err,
-                            cudaStream_t st, TcEvents& ev, std::string* why) {
+                            cudaStream_t st, TcEvents& ev, std::string* why, unsigned ready) {
     const int group = tc_group_of(tile_cfg);
     // bits 0-1: 1 = 128, 2 = 256 columns per tile; bit 3: CTA pairs (256 rows); default (0):
     // 256 x 256 tiles on CTA pairs
@@ -1927,19 +2039,11 @@ cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const floa
     uint8_t* base = static_cast<uint8_t*>(scratch);
     uint8_t *qa = base + L.qa, *qb = base + L.qb;
     uint8_t *sa = base + L.sa, *sb = base + L.sb;
-    {
-        const int64_t warps = L.Mp * L.kbs;
-        int64_t g = (warps * 32 + 255) / 256;
-        if (g > (int64_t)sm_count() * 8) g = (int64_t)sm_count() * 8;
-        quant_rows_fp8_kernel<<<(unsigned)g, 256, 0, st>>>(A, M, K, L.Mp, L.Kp, qa, sa);
-        cudaError_t e = cudaGetLastError();
+    for (int which = 0; which < 2; ++which) {
+        if (ready & (1u << which)) continue;  // formed by tc_init_planes
+        const cudaError_t e = quant_fp8<false>(which, which == 0 ? A : B, InitSrc{}, M, N, K, base, st);
         if (e != cudaSuccess) return e;
-        dim3 grid((unsigned)(L.Np / kQuantCols), (unsigned)L.kbs);
-        if (grid.y > 65535u) return cudaErrorInvalidValue;
-        quant_cols_fp8_kernel<<<grid, 256, 0, st>>>(B, K, N, L.Np, L.Kp, qb, sb);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        ev.launches += 2;
+        ev.launches += 1;
     }
     CUtensorMap ta, tb;
     if (!make_map(&ta, qa, L.Kp, L.Mp, BM, true, why)) return cudaErrorInvalidValue;
@@ -2036,16 +2140,10 @@ cudaError_t tc_prepare(int prec, float* C, const float* A, const float* B, const
         uint8_t* base = static_cast<uint8_t*>(scratch);
         uint8_t *qa = base + L.qa, *qb = base + L.qb;
         uint8_t *sa = base + L.sa, *sb = base + L.sb;
-        const int64_t warps = L.Mp * L.kbs;
-        int64_t g = (warps * 32 + 255) / 256;
-        if (g > (int64_t)sm_count() * 8) g = (int64_t)sm_count() * 8;
-        quant_rows_fp8_kernel<<<(unsigned)g, 256, 0, st>>>(A, M, K, L.Mp, L.Kp, qa, sa);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        dim3 grid((unsigned)(L.Np / kQuantCols), (unsigned)L.kbs);
-        if (grid.y > 65535u) return cudaErrorInvalidValue;
-        quant_cols_fp8_kernel<<<grid, 256, 0, st>>>(B, K, N, L.Np, L.Kp, qb, sb);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        for (int which = 0; which < 2; ++which) {
+            const cudaError_t e = quant_fp8<false>(which, which == 0 ? A : B, InitSrc{}, M, N, K, base, st);
+            if (e != cudaSuccess) return e;
+        }
         *launches = 2;
         if (!make_map(&prob->ta, qa, L.Kp, L.Mp, BM, true, why)) return cudaErrorInvalidValue;
         if (!make_map(&prob->tb, qb, L.Kp, L.Np, 128, true, why)) return cudaErrorInvalidValue;

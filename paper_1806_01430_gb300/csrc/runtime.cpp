@@ -1603,8 +1603,8 @@ double ev_ms(cudaEvent_t a, cudaEvent_t b) {
 // kernels (or its host loop), the outputs' copies back and the error word's read-back.
 // When every loop is on the GPU this is also what a CUDA graph of the run captures.
 // The GEMM loop that alone reads INIT loop li's output b, as its A (*which = 0) or its B
-// (*which = 1), when that GEMM runs on the GPU in split bfloat16: b is then formed straight
-// into the GEMM's bfloat16 planes, never as binary32.  A GEMM with its chain takes operands of
+// (*which = 1), when that GEMM runs on the tensor cores: b is then formed straight into the
+// GEMM's bfloat16 planes or e4m3 codes, never as binary32.  A GEMM with its chain takes operands of
 // at least kPlanesMinBytes this way; below that the split it saves is a few us.  Whole pass:
 // six-loop program 4096, three terms, B: 664 -> 643 us; twelve-loop 6000, K = 1500, two terms, A
 // and B: 455 -> 435.  -1 otherwise (b is not a TEMP buffer, is read by anything else or written
@@ -1614,7 +1614,7 @@ int planes_consumer(const gao_prog* p, int li, int b, uint64_t gene_mask, bool f
     const BufState& B = p->bufs[(size_t)b];
     if (B.d.role != GAO_BUF_TEMP || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT || p->lay.tc_bytes == 0) return -1;
     const int prec = p->opts.gemm_prec;
-    if (prec != GAO_GEMM_BF16 && prec != GAO_GEMM_BF16X3 && prec != GAO_GEMM_BF16X6) return -1;
+    if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_FP8) return -1;
     int reader = -1, gemms = 0;
     for (int j = 0; j < (int)p->loops.size(); ++j) {
         const gao_loop& Lj = p->loops[(size_t)j];

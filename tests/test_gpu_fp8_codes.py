@@ -59,3 +59,25 @@ def test_codes_of_both_operands(gao, m, k):
         C = gao.prog_output(p, 3)
         assert np.array_equal(C if A is X else C.T, want)
         gao.prog_destroy(p)
+
+
+@pytest.mark.parametrize("rowscale", [0, 3])
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (5, 63, 129), (130, 64, 127), (129, 201, 256), (300, 65, 385), (257, 1001, 1030)])
+def test_codes_formed_by_the_init_loop(gao, m, n, k, rowscale):
+    """A and B formed straight as codes (TEMP) against INIT then quantisation (kept as OUTPUT), with
+    and without rows scaled: the same bits of C."""
+    got = []
+    for keep in (False, True):
+        role = W.OUTPUT if keep else W.TEMP
+        bufs = [W.Buffer("A", m, k, role=role), W.Buffer("B", k, n, role=role), W.Buffer("C0", m, n),
+                W.Buffer("C", m, n, role=W.OUTPUT)]
+        loops = [W.Loop(W.INIT, [], [0, 1, 2], flags=rowscale), W.Loop(W.GEMM, [0, 1, 2], [3], 1.5, 0.5)]
+        p = gao.prog_create(bufs, loops, seed=m + n + k, gemm_prec=gao.FP8)
+        for _ in range(3):  # plain, captured, replayed
+            gao.prog_run(p, 0b11)
+            got.append(gao.prog_output(p, 3))
+            assert [gao.prog_planes_for(p, b) for b in (0, 1)] == ([-1, -1] if keep else [1, 1])
+            assert gao.prog_stats(p)[1]["launches"] == (3 if keep else 1)
+        gao.prog_destroy(p)
+    for c in got:
+        assert np.array_equal(c.view(np.uint32), got[-1].view(np.uint32))
