@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <array>
 #include <unordered_map>
 #include <vector>
 
@@ -49,7 +50,7 @@ struct GraphEntry {
     bool failed = false;
     cudaGraphExec_t exec = nullptr;
     std::vector<uint8_t> vh, vd;
-    std::vector<int> gen_chain;
+    std::vector<std::array<int, 4>> gen;  // the buffers' gen_loop, gen_slot, gen_for, gen_chain
     std::vector<gao_loop_stat> stats;
     std::vector<uint8_t> ev_used;
 };

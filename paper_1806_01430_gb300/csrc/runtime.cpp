@@ -2031,11 +2031,12 @@ void capture_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags, Graph
         ge->exec = exec;
         ge->vh.resize(p->bufs.size());
         ge->vd.resize(p->bufs.size());
-        ge->gen_chain.resize(p->bufs.size());
+        ge->gen.resize(p->bufs.size());
         for (size_t b = 0; b < p->bufs.size(); ++b) {
             ge->vh[b] = p->bufs[b].vh;
             ge->vd[b] = p->bufs[b].vd;
-            ge->gen_chain[b] = p->bufs[b].gen_chain;
+            const BufState& B = p->bufs[b];
+            ge->gen[b] = {B.gen_loop, B.gen_slot, B.gen_for, B.gen_chain};
         }
         ge->stats = p->stats;
         ge->ev_used = p->ev_used;
@@ -2092,7 +2093,11 @@ extern "C" gao_status prog_run(gao_prog* p, uint64_t gene, uint32_t flags, doubl
         for (size_t b = 0; b < p->bufs.size(); ++b) {
             p->bufs[b].vh = ge->vh[b] != 0;
             p->bufs[b].vd = ge->vd[b] != 0;
-            p->bufs[b].gen_chain = ge->gen_chain[b];
+            BufState& B = p->bufs[b];
+            B.gen_loop = ge->gen[b][0];
+            B.gen_slot = ge->gen[b][1];
+            B.gen_for = ge->gen[b][2];
+            B.gen_chain = ge->gen[b][3];
         }
         p->run_mask = gene_mask;
         p->run_fuse = fuse;
