@@ -243,8 +243,9 @@ gao_status prog_device_ptr(gao_prog *p, int buf, void **dev_ptr);
 
 /* INIT into GEMM operand planes: a TEMP buffer that an INIT loop writes and that only one
  * GEMM reads -- as its A or B, on the tensor cores, with resident transfers and no other GEMM
- * on the GPU; for a GEMM with a fused chain, of at least 16 MiB, with A on the device -- is
- * formed by the INIT loop straight into that GEMM's bfloat16 planes or e4m3 codes (the counter
+ * on the GPU; for a GEMM with a fused chain, of at least 16 MiB, with A on the device when the
+ * GEMM runs; beside an A that comes from the host in row blocks, never -- is formed by the
+ * INIT loop straight into that GEMM's bfloat16 planes or e4m3 codes (the counter
  * hash's values split or quantised as the GEMM's own kernels would; the GEMM then skips
  * them), and its binary32 array is not written.  *gemm_loop = that GEMM loop if the
  * last run formed buffer `buf` this way and nothing has formed its binary32 values since,

@@ -1237,16 +1237,24 @@ gao_status run_gpu_chain(RunCtx& R, int li, const Chain& ch) {
 // start as soon as its rows have landed, while the next block is still on the link.  Row
 // blocks and column ranges give the same bits as one launch (every output is formed the
 // same way); only the split precisions take this path.
-int64_t pipeline_blocks(const gao_prog* p, const gao_loop& L) {
+// The row blocks of GEMM loop L when its A has to come (0: it is not run this way).
+int64_t row_blocks(const gao_prog* p, const gao_loop& L) {
     const int prec = p->opts.gemm_prec;
     if (L.kind != GAO_LOOP_GEMM) return 0;
     if (prec != GAO_GEMM_BF16 && prec != GAO_GEMM_BF16X3 && prec != GAO_GEMM_BF16X6) return 0;
     if (L.ins[0] == L.ins[1] || L.ins[2] == L.ins[0] || L.ins[2] == L.ins[1]) return 0;
     const BufState& A = p->bufs[(size_t)L.ins[0]];
     const gao_buffer& B = p->bufs[(size_t)L.ins[1]].d;
-    if (A.vd || A.gen_for >= 0 || A.bytes < kPipelineMinBytes || A.d.cols <= 0 || B.cols <= 0) return 0;
+    if (A.bytes < kPipelineMinBytes || A.d.cols <= 0 || B.cols <= 0) return 0;
     const int64_t blocks = std::min<int64_t>(kMaxRowBlocks, A.d.rows / 256);
     return blocks >= 2 ? blocks : 0;
+}
+
+// Row blocks split their operands themselves: operands formed as planes are read whole.
+int64_t pipeline_blocks(const gao_prog* p, const gao_loop& L) {
+    if (L.kind != GAO_LOOP_GEMM) return 0;
+    const BufState &A = p->bufs[(size_t)L.ins[0]], &B = p->bufs[(size_t)L.ins[1]];
+    return A.vd || A.gen_for >= 0 || B.gen_for >= 0 ? 0 : row_blocks(p, L);
 }
 
 // With early_out (C an OUTPUT the run copies back at its end), each block's rows of C go back
@@ -1632,13 +1640,16 @@ int planes_consumer(const gao_prog* p, int li, int b, uint64_t gene_mask, bool f
     const gao_loop& G = p->loops[(size_t)reader];
     if (G.kind != GAO_LOOP_GEMM || !((gene_mask >> reader) & 1)) return -1;
     if (G.outs[0] == b || G.ins[2] == b || (G.ins[0] == b) == (G.ins[1] == b)) return -1;
+    // whether A will be on the device when the GEMM runs, as the last loop before it that writes A
+    // leaves it (this loop: on the device); A still to come from the host runs in row blocks where it
+    // is large enough, which split their operands
+    bool a_here = p->bufs[(size_t)G.ins[0]].vd;
+    for (int j = li; j < reader; ++j)
+        for (int o : loop_outputs(p->loops[(size_t)j]))
+            if (o == G.ins[0]) a_here = (gene_mask >> j) & 1;
+    if (!a_here && row_blocks(p, G) > 0) return -1;
     Chain c;
-    if (find_chain(p, reader, gene_mask, fuse, &c)) {
-        // A still to come from the host would run in row blocks, which split their operands
-        const std::vector<int> mine = loop_outputs(p->loops[(size_t)li]);
-        const bool a_here = p->bufs[(size_t)G.ins[0]].vd || std::find(mine.begin(), mine.end(), G.ins[0]) != mine.end();
-        if (B.bytes < kPlanesMinBytes || !a_here) return -1;
-    }
+    if (find_chain(p, reader, gene_mask, fuse, &c) && (B.bytes < kPlanesMinBytes || !a_here)) return -1;
     const gao_buffer &A = p->bufs[(size_t)G.ins[0]].d, &Bm = p->bufs[(size_t)G.ins[1]].d;
     if (A.rows <= 0 || A.cols <= 0 || Bm.cols <= 0) return -1;
     *which = G.ins[0] == b ? 0 : 1;
