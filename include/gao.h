@@ -238,16 +238,19 @@ gao_status prog_output(gao_prog *p, int buf, const void **host_ptr, gao_buffer *
 /* Device pointer of buffer `buf` (for callers that keep data on the GPU).  A buffer the
  * last run formed only as a GEMM's bfloat16 planes (prog_planes_for), or reduced without
  * writing it (fuse_chains), gets its binary32 values formed first (the INIT slot or the
- * element-wise chain alone, on the program's stream, waited for). */
+ * element-wise chain alone, on the program's stream, waited for).  From the first call for
+ * `buf` on, every run writes the array itself, so a pointer that is kept from run to run
+ * sees each run's values. */
 gao_status prog_device_ptr(gao_prog *p, int buf, void **dev_ptr);
 
-/* INIT into GEMM operand planes: a TEMP buffer that an INIT loop writes and that only one
- * GEMM reads -- as its A or B, on the tensor cores, with resident transfers and no other GEMM
- * on the GPU; for a GEMM with a fused chain, of at least 16 MiB, with A on the device when the
- * GEMM runs; beside an A that comes from the host in row blocks, never -- is formed by the
- * INIT loop straight into that GEMM's bfloat16 planes or e4m3 codes (the counter
- * hash's values split or quantised as the GEMM's own kernels would; the GEMM then skips
- * them), and its binary32 array is not written.  *gemm_loop = that GEMM loop if the
+/* INIT into GEMM operand planes: a TEMP buffer that an INIT loop writes, that only one GEMM
+ * reads, as its A or B, on the tensor cores, and whose device pointer nobody has asked for
+ * (prog_device_ptr) is formed by the INIT loop straight into that GEMM's bfloat16 planes or
+ * e4m3 codes (the counter hash's values split or quantised as the GEMM's own kernels would;
+ * the GEMM then skips them), and its binary32 array is not written.  This takes resident
+ * transfers, no other GEMM on the GPU and no A that the GEMM copies from the host in row
+ * blocks; for a GEMM with a fused chain also an operand of at least 16 MiB and an A that is on
+ * the device when the GEMM runs.  *gemm_loop = that GEMM loop if the
  * last run formed buffer `buf` this way and nothing has formed its binary32 values since,
  * else -1.  Anything that reads the buffer afterwards (prog_gemm_residual, prog_device_ptr,
  * prog_autotune) forms it from the INIT slot first. */

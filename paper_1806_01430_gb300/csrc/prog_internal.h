@@ -26,6 +26,9 @@ struct BufState {
     // The last value of the element-wise chain that starts at this loop, which the last run
     // reduced without writing it: prog_device_ptr forms it (vd and vh false until then).
     int gen_chain = -1;
+    // The caller has taken the device pointer: every later run writes the array itself (neither
+    // of the two above), since what the pointer is read for afterwards cannot be known.
+    bool held = false;
 };
 
 struct CacheEntry {

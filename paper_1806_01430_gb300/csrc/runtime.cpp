@@ -1079,7 +1079,7 @@ bool find_ew_chain(const gao_prog* p, int li, uint64_t mask, bool fuse, EwPlan* 
     }
     const int last = e.loops[e.n - 1];
     const BufState& P = p->bufs[(size_t)cur];
-    if (P.d.role != GAO_BUF_OUTPUT && ew_chain_reduce_fits(P.d.rows, P.d.cols)) {
+    if (P.d.role != GAO_BUF_OUTPUT && !P.held && ew_chain_reduce_fits(P.d.rows, P.d.cols)) {
         int sum = -1, colmax = -1, j = last + 1;
         for (; j < n && ((mask >> j) & 1); ++j) {
             const gao_loop& R = p->loops[(size_t)j];
@@ -1616,11 +1616,11 @@ double ev_ms(cudaEvent_t a, cudaEvent_t b) {
 // at least kPlanesMinBytes this way; below that the split it saves is a few us.  Whole pass:
 // six-loop program 4096, three terms, B: 664 -> 643 us; twelve-loop 6000, K = 1500, two terms, A
 // and B: 455 -> 435.  -1 otherwise (b is not a TEMP buffer, is read by anything else or written
-// by another loop, the GEMM reads it twice or also as C0, another GEMM on the GPU uses the one
-// room for planes, transfers are per loop).
+// by another loop, the caller holds its device pointer, the GEMM reads it twice or also as C0,
+// another GEMM on the GPU uses the one room for planes, transfers are per loop).
 int planes_consumer(const gao_prog* p, int li, int b, uint64_t gene_mask, bool fuse, int* which) {
     const BufState& B = p->bufs[(size_t)b];
-    if (B.d.role != GAO_BUF_TEMP || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT || p->lay.tc_bytes == 0) return -1;
+    if (B.d.role != GAO_BUF_TEMP || B.held || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT || p->lay.tc_bytes == 0) return -1;
     const int prec = p->opts.gemm_prec;
     if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_FP8) return -1;
     int reader = -1, gemms = 0;
@@ -2160,6 +2160,14 @@ extern "C" gao_status prog_device_ptr(gao_prog* p, int buf, void** dev_ptr) {
         gao_status s = B.gen_chain >= 0 ? form_chain_value(R, buf) : materialize(R, buf);
         if (s != GAO_OK) return s;
         if ((ce = cudaStreamSynchronize(p->st)) != cudaSuccess) return cuda_fail(ce, "cudaStreamSynchronize");
+    }
+    if (!B.held) {
+        B.held = true;
+        for (const auto& kv : p->graphs)  // captured runs that leave the array unwritten
+            if (kv.second.exec && (kv.second.gen[(size_t)buf][0] >= 0 || kv.second.gen[(size_t)buf][3] >= 0)) {
+                drop_graphs(p);
+                break;
+            }
     }
     *dev_ptr = B.dev;
     return GAO_OK;
