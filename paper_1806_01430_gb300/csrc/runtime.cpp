@@ -2448,6 +2448,10 @@ extern "C" gao_status prog_autotune(gao_prog* p, const gao_ga_params* params, ga
         gao_loop_stat dummy{};
         for (int b : {L.ins[0], L.ins[1]})
             if ((st = make_valid(R, b, true, dummy)) != GAO_OK) return st;
+        // ... and the values that the run only reduced, before the timed launches change what
+        // they are formed from (C, and with a chain D and E)
+        for (size_t b = 0; b < p->bufs.size(); ++b)
+            if (p->bufs[b].gen_chain >= 0 && (st = form_chain_value(R, (int)b)) != GAO_OK) return st;
     }
     const gao_buffer &A = p->bufs[(size_t)L.ins[0]].d, &B = p->bufs[(size_t)L.ins[1]].d;
     float* C = (float*)p->bufs[(size_t)L.outs[0]].dev;
