@@ -441,6 +441,7 @@ gao_status run_genes(gao_batch* b, const uint64_t* genes, int u, double* seconds
             for (auto& B : p->bufs) {
                 B.vh = (B.d.role == GAO_BUF_INPUT);
                 B.vd = false;
+                B.gen_loop = B.gen_slot = B.gen_for = B.gen_chain = -1;  // of a run of the program alone
             }
             rc[(size_t)r].push_back(RunCtx{p, 0.0, false, CpuCtx{p->opts.cpu_threads, 0.0, false}, b->st, false});
         }

@@ -74,3 +74,17 @@ def test_kept_pointer_sees_every_run(gao, case, before):
             assert torch.equal(held[b], want[b]), b
             assert gao.prog_planes_for(p, b) == -1
     gao.prog_destroy(p)
+
+
+def test_batch_run_ends_the_planes_of_a_run_alone(gao):
+    """A batch writes binary32 operands: what an earlier run of the program formed as planes is
+    not reported, or formed again, after it."""
+    bufs, loops = gemm(200, 129, 300)
+    p = gao.prog_create(bufs, loops, seed=7, gemm_prec=BF16X3)
+    gao.prog_run(p, 0b11)
+    assert [gao.prog_planes_for(p, b) for b in (0, 1)] == [1, 1]
+    b = gao.batch_create([p])
+    gao.batch_evaluate(b, [0b11])
+    assert [gao.prog_planes_for(p, i) for i in (0, 1)] == [-1, -1]
+    gao.batch_destroy(b)
+    gao.prog_destroy(p)
