@@ -527,7 +527,7 @@ gao_status gao_selftest_device_wait(double limit_s, void *stream);
  * (which may synchronise the device and can fail with out-of-memory mid-run).
  *
  * It allocates nothing and calls no allocating routine.  One kernel forms the maxima
- * in shared memory; tall inputs of few columns need scratch, one 32-bit key per column,
+ * in shared memory; tall and large inputs need scratch, one 32-bit key per column,
  * a fixed array of GAO_COLMAX_NOALLOC_MAX_COLS keys (256 KiB) inside
  * the library; every GPU that loads the library holds that array until the process
  * exits.  cols above the maximum is rejected with GAO_EINVAL.  The first call on a

@@ -142,7 +142,7 @@ cudaError_t launch_frobenius(double* out, const float* in, int64_t n, ReduceScra
 cudaError_t launch_sum(double* out, const float* in, int64_t n, ReduceScratch rs, cudaStream_t st);
 cudaError_t launch_relu(float* out, const float* in, int64_t n, cudaStream_t st);
 cudaError_t launch_square(float* out, const float* in, int64_t n, cudaStream_t st);
-// keys: scratch of cols words, used for tall inputs of few columns only; *launches: kernels issued.
+// keys: scratch of cols words, used for tall and large inputs only; *launches: kernels issued.
 cudaError_t launch_colmax(float* out, const float* in, int64_t rows, int64_t cols, uint32_t* keys, cudaStream_t st,
                           int* launches = nullptr);
 // Output rows [row_begin, row_end) of the rows x cols image (row_end < 0: to the last row);

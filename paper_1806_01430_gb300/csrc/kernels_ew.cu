@@ -558,8 +558,8 @@ __global__ void __launch_bounds__(256) reduce64_kernel(double* __restrict__ out,
 // strip (16 bytes per lane where rows are 16-byte aligned, else four strided words), kColAhead
 // rows' loads in flight per thread; the order-preserving integer keys are reduced over the
 // block in shared memory and over the cluster in its first block, which decodes and stores.
-// Bound by HBM for large inputs and by launch latency for small ones.  It replaces, wherever the
-// columns are many enough to fill the GPU this way, keys in global memory (cleared by a
+// Bound by HBM for large inputs and by launch latency for small ones.  It replaces, within the
+// sizes of colmax_in_strips, keys in global memory (cleared by a
 // memset, raised by one atomic per column and row chunk, decoded by another launch): 1080 x 1920
 // 29.7 -> 6.5 us, 4096 x 4096 26.7 -> 10.7 us (6.3 TB/s), 8192 x 8192 54.4 -> 45.7 us.
 constexpr int kColAhead = 8;
@@ -636,8 +636,8 @@ __global__ void __launch_bounds__(256) colmax_strip_kernel(float* __restrict__ o
 
 // Column maxima via order-preserving integer keys and atomicMax (max is exact and
 // order-free, so the result is deterministic).  Thread = 4 consecutive columns of
-// a chunk of rows.  For tall inputs of few columns, whose rows must spread over more blocks
-// than a cluster holds.
+// a chunk of rows.  For the inputs that colmax_in_strips leaves: tall ones, whose rows must
+// spread over more blocks than a cluster holds, and large ones.
 __global__ void colmax_keys_kernel(uint32_t* __restrict__ keys, const float* __restrict__ in, int64_t rows,
                                    int64_t cols, int64_t rows_per_chunk) {
     const int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4;
@@ -1508,8 +1508,35 @@ cudaLaunchConfig_t strip_config(int64_t cols, int vx, int cluster, cudaStream_t 
 }
 }  // namespace
 
+namespace {
+// Whether column maxima run in strips; else by the keys kernels, whose launches cost ~30 us in all
+// but which read whole rows over the whole GPU.  Strips against keys, us, L2 flushed:
+//  - 16-byte aligned rows: strips up to 65536 rows and 2^26 values (65536 x 300 74 / 75, 80000 x 300
+//    91 / 82, 400000 x 300 369 / 161, 80000 x 600 95 / 92, 65536 x 1000 83 / 100, 120000 x 1000 136 /
+//    132, 8192 x 8192 62 / 64, 16384 x 19456 232 / 212, and the closest loss 3400 x 19456 67 / 64);
+//    wide strips that make fewer than three blocks an SM, too little in flight, up to 3 x 2^24
+//    (8192 x 4900 50 / 51, 12000 x 4900 66 / 63, 32768 x 4900 146 / 125);
+//  - rows of any other alignment, which the keys kernel reads a word at a time: always strips
+//    (131072 x 301 74 / 125, 1000000 x 301 453 / 532, 200000 x 2401 414 / 466);
+//  - up to 16 columns, where the eight blocks of one strip are all there is: up to 8192 rows
+//    (8192 x 4 13 / 14, 16384 x 4 19 / 16, 16384 x 8 21 / 16; 16384 x 32 21 / 24).
+bool colmax_in_strips(int64_t rows, int64_t cols, bool vec, int* vx, int* cluster) {
+    if (!strip_plan(rows, cols, INT64_MAX, vx, cluster)) return false;
+    if (cols <= 16 && rows > 8192) return false;
+    if (!vec) return true;
+    const int64_t blocks = (cols + 4 * *vx - 1) / (4 * *vx) * *cluster;
+    const bool few = *vx > 8 && blocks < 3 * (int64_t)sm_count();
+    return rows <= 65536 && rows * cols <= (int64_t)(few ? 3 : 4) << 24;
+}
+}  // namespace
+
 bool ew_chain_reduce_fits(int64_t rows, int64_t cols) {
     int vx, cluster;
+    // fewer than three blocks for five SMs lose to the separate passes where the launches saved
+    // no longer count: 131072 x 300 178 us against 189, 200000 x 289 292 / 297, but 266666 x 300 343 /
+    // 337 and 276816 x 289 395 / 389; 12 strips (227272 x 352 has 11) gain at any height
+    const int64_t strips = (cols + 31) / 32;
+    if (strips * 8 * 5 < 3 * (int64_t)sm_count() && rows > 131072) return false;
     return strip_plan(rows, cols, reduce_blocks(), &vx, &cluster);
 }
 
@@ -1534,8 +1561,8 @@ cudaError_t launch_colmax(float* out, const float* in, int64_t rows, int64_t col
     if (launches) *launches = 0;
     if (cols <= 0) return cudaSuccess;
     int vx, cluster;
-    if (strip_plan(rows, cols, INT64_MAX, &vx, &cluster)) {
-        const bool vec = (cols % 4 == 0) && ((uintptr_t)in & 15u) == 0;
+    const bool vec = (cols % 4 == 0) && ((uintptr_t)in & 15u) == 0;
+    if (colmax_in_strips(rows, cols, vec, &vx, &cluster)) {
         cudaLaunchAttribute at;
         const cudaLaunchConfig_t lc = strip_config(cols, vx, cluster, st, &at);
         auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, out, in, rows, cols, cluster); };
