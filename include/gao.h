@@ -531,8 +531,9 @@ gao_status gao_selftest_device_wait(double limit_s, void *stream);
  * a fixed array of GAO_COLMAX_NOALLOC_MAX_COLS keys (256 KiB) inside
  * the library; every GPU that loads the library holds that array until the process
  * exits.  cols above the maximum is rejected with GAO_EINVAL.  The first call on a
- * device (with that device current) looks up the array's device address; make that
- * first call before any stream capture.  A call that uses the keys clears them on
+ * device (with that device current) looks up the array's device address and loads every
+ * kernel that a later call of any shape may run; make that first call before any stream
+ * capture.  A call that uses the keys clears them on
  * `stream` before reducing, and all calls share the one array: calls whose work
  * overlaps on the GPU (different streams, or several host threads) may race and give
  * wrong results.  Asynchronous on `stream` (NULL: the legacy default stream);

@@ -1864,6 +1864,15 @@ cudaError_t colmax_noalloc_keys(uint32_t** out) {
         void* p = nullptr;
         e = cudaGetSymbolAddress(&p, g_colmax_noalloc_keys);
         if (e != cudaSuccess) return e;
+        // kernels load when first used (which may allocate, and wait for the device): all that a
+        // later call can take, whatever its shape and alignment, load now
+        for (const void* k : {(const void*)colmax_strip_kernel<8, false>, (const void*)colmax_strip_kernel<8, true>,
+                              (const void*)colmax_strip_kernel<16, false>, (const void*)colmax_strip_kernel<16, true>,
+                              (const void*)colmax_strip_kernel<32, false>, (const void*)colmax_strip_kernel<32, true>,
+                              (const void*)colmax_keys_kernel, (const void*)colmax_decode_kernel}) {
+            cudaFuncAttributes a;
+            if ((e = cudaFuncGetAttributes(&a, k)) != cudaSuccess) return e;
+        }
         g_noalloc_keys_dev[dev] = static_cast<uint32_t*>(p);
     }
     *out = g_noalloc_keys_dev[dev];
