@@ -394,7 +394,8 @@ gao_status prog_autotune(gao_prog *p, const gao_ga_params *params, gao_autotune_
  * new genes of a population or GA generation are measured up to R at a time: gene r runs
  * on copy r, the copies' phases go one after another on the batch's stream, and the
  * GEMMs of every one of these genes that offloads the GEMM loop -- genes x programs --
- * run in ONE grouped persistent launch.  Since genes share that launch, a gene's time is
+ * run in ONE grouped persistent launch (the genes with the chain in the epilogue in one of
+ * their own where the suite's sizes give those another kernel).  Since genes share that launch, a gene's time is
  * attributed: the device time of its own phase graphs and boundary copies (CUDA events
  * around each), the span of its own problems inside the grouped launch (global-timer
  * stamps taken by the kernel when it starts a tile's loads and when it has stored a tile),
@@ -409,12 +410,12 @@ typedef struct gao_batch_stat {
     int64_t executed;          /* genes measured                                        */
     int64_t served;            /* genes answered from the cache                         */
     double exec_seconds;       /* host wall time spent measuring genes                  */
-    double gemm_phase_ms;      /* GPU time of the last grouped GEMM launch (events around
-                                  it; the operand splits are part of the GEMM loop's
+    double gemm_phase_ms;      /* GPU time of the last gene group's grouped GEMM launches (events
+                                  around them; the operand splits are part of the GEMM loop's
                                   phase graph before it)                                 */
-    double gemm_flops;         /* 2MNK summed over that launch's GEMMs (over the suite
+    double gemm_flops;         /* 2MNK summed over those launches' GEMMs (over the suite
                                   before any launch)                                     */
-    int32_t gemm_tiles;        /* CTAs (output tiles) of that launch                    */
+    int32_t gemm_tiles;        /* CTAs (output tiles) of those launches                 */
     int32_t launches_per_gene; /* kernels the all-GPU gene launches                     */
     int32_t graphs;            /* phase graphs captured for the suite                   */
     int32_t fused_phases;      /* GEMM phases run with the loop chain in the epilogue

@@ -78,6 +78,7 @@ struct gao_batch {
     std::vector<cudaEvent_t> ev;    // [replica][loop][kEv], then [replica][2] for the final copies
     int gemm_loop = -1;
     bool grouped_gemm = false;
+    bool wide_chains = false;       // problems with a chain run in a launch of sixteen epilogue warps
     bool chunked = false;           // some program restarts its accumulators every K chunk
     int init_loop = -1;             // INIT loop run as one grouped launch over all programs
     int n_init = 0;
@@ -268,7 +269,7 @@ gao_status make_chain(gao_batch* b, Replica& R, uint64_t mask, const Chain& ch, 
         int64_t M, N, K;
         gemm_shape(p, b->gemm_loop, &M, &N, &K);
         int nl = 0;
-        e = tc_finalize_chain(b->prec, M, N, K, p->arena + p->lay.tc_off, fz[j], b->side[j % kSide], &nl);
+        e = tc_finalize_chain(b->prec, M, N, K, p->arena + p->lay.tc_off, fz[j], b->wide_chains, b->side[j % kSide], &nl);
         cv->kernels += nl;
     }
     if (e == cudaSuccess) e = join_side(b);
@@ -371,21 +372,22 @@ gao_status size_tables(gao_batch* b, int reps) {
     return GAO_OK;
 }
 
-// One grouped launch over the GEMM problems of the replicas in `parts` (their plain
-// problems, or a chain variant's where cv[r] is set), in that order; with `spans` every
-// problem's time span is recorded and copied to h_span (stream order).
+// One grouped launch over the GEMM problems of the replicas in `parts` (their plain problems,
+// or a chain variant's where cv[r] is set), in that order; with wide chains a second one takes
+// the replicas with a chain, which come last.  With `spans` every problem's time span is recorded
+// and copied to h_span (stream order).
 gao_status grouped_launch(gao_batch* b, const std::vector<int>& parts, const std::vector<ChainVar*>& cv, bool spans) {
     GAO_CUDA_TRY(cudaEventSynchronize(b->tab_ev));  // the previous table copy has read h_table
-    int k = 0, start = 0;
-    bool chain = false;
+    int k = 0, probs[2] = {0, 0}, tiles[2] = {0, 0};  // of the launches with eight and sixteen epilogue warps
     for (int r : parts) {
-        chain |= cv[(size_t)r] != nullptr;
+        const int w = b->wide_chains && cv[(size_t)r] ? 1 : 0;
         const std::vector<TcProblem>& src = cv[(size_t)r] ? cv[(size_t)r]->probs : b->reps[(size_t)r].probs;
         for (const TcProblem& pr : src) {
-            if (k >= b->table_cap) return fail(GAO_EINVAL, "batch problem table overflow");
+            if (k >= b->table_cap || (w == 0 && probs[1] > 0)) return fail(GAO_EINVAL, "batch problem table overflow");
             TcProblem t = pr;
-            t.tile_start = start;
-            start += t.tiles_m * t.tiles_n;
+            t.tile_start = tiles[w];
+            tiles[w] += t.tiles_m * t.tiles_n;
+            probs[w] += 1;
             t.span_start = spans ? b->d_span + k : nullptr;
             t.span_end = spans ? b->d_span + b->table_cap + k : nullptr;
             b->h_table[k++] = t;
@@ -398,7 +400,13 @@ gao_status grouped_launch(gao_batch* b, const std::vector<int>& parts, const std
         GAO_CUDA_TRY(cudaMemsetAsync(b->d_span + b->table_cap, 0, sizeof(unsigned long long) * (size_t)k, b->st));
     }
     GAO_CUDA_TRY(cudaEventRecord(b->g0, b->st));
-    GAO_CUDA_TRY(tc_launch_grouped(b->prec, b->chunked, chain, b->d_probs, k, start, b->d_err, b->st));
+    int launches = 0;
+    for (int w = 0; w < 2; ++w) {
+        if (probs[w] == 0) continue;
+        GAO_CUDA_TRY(tc_launch_grouped(b->prec, b->chunked, w == 1, b->d_probs + (w ? probs[0] : 0), probs[w], tiles[w],
+                                       b->d_err, b->st));
+        launches += 1;
+    }
     GAO_CUDA_TRY(cudaEventRecord(b->g1, b->st));
     if (spans) {
         GAO_CUDA_TRY(cudaMemcpyAsync(b->h_span, b->d_span, sizeof(unsigned long long) * (size_t)k,
@@ -406,10 +414,10 @@ gao_status grouped_launch(gao_batch* b, const std::vector<int>& parts, const std
         GAO_CUDA_TRY(cudaMemcpyAsync(b->h_span + b->table_cap, b->d_span + b->table_cap,
                                      sizeof(unsigned long long) * (size_t)k, cudaMemcpyDeviceToHost, b->st));
     }
-    b->stat.kernel_launches += 1;
-    b->stat.grouped_launches += 1;
+    b->stat.kernel_launches += launches;
+    b->stat.grouped_launches += launches;
     b->stat.grouped_genes += (int64_t)parts.size();
-    b->stat.gemm_tiles = start;
+    b->stat.gemm_tiles = tiles[0] + tiles[1];
     b->stat.gemm_flops = b->flops_per_suite * (double)parts.size();
     return GAO_OK;
 }
@@ -521,7 +529,10 @@ gao_status run_genes(gao_batch* b, const uint64_t* genes, int u, double* seconds
             }
         }
         if (!parts.empty()) {
-            // every offloaded GEMM of these genes' suites in one grouped launch
+            // every offloaded GEMM of these genes' suites in one grouped launch (two with wide chains
+            // beside genes without a chain)
+            if (b->wide_chains)
+                std::stable_partition(parts.begin(), parts.end(), [&](int r) { return cv[(size_t)r] == nullptr; });
             for (size_t k = 0; k < parts.size(); ++k) part_index[(size_t)parts[k]] = (int)k;
             gao_status s = grouped_launch(b, parts, cv, attributed);
             if (s != GAO_OK) return s;
@@ -733,18 +744,21 @@ extern "C" gao_status batch_create(gao_prog* const* progs, int n_progs, gao_batc
     if (b->grouped_gemm) {
         std::string why;
         if (!tc_available(&why)) return bail(fail(GAO_ENODEV, why));
-        for (bool chain : {false, true})
-            if ((e = tc_launch_grouped(b->prec, b->chunked, chain, nullptr, 0, 0, nullptr, b->st)) != cudaSuccess)
-                return bail(cuda_fail(e, "grouped GEMM set-up"));
-        int64_t start = 0;
+        int64_t start = 0, unaligned = 0;
         for (int i = 0; i < n_progs; ++i) {
             int64_t m, nn, k;
             gemm_shape(progs[i], b->gemm_loop, &m, &nn, &k);
             if (m <= 0 || nn <= 0 || k <= 0)
                 return bail(fail(GAO_EINVAL, "batch GEMM needs positive sizes on the tensor-core path"));
             b->flops_per_suite += 2.0 * m * nn * k;
-            start += ((m + 127) / 128) * ((nn + 127) / 128);
+            const int64_t tiles = ((m + 127) / 128) * ((nn + 127) / 128);
+            start += tiles;
+            if (nn % 4 != 0) unaligned += tiles;
         }
+        b->wide_chains = b->fuse && tc_grouped_wide(b->prec, start, unaligned);
+        for (int w = 0; w <= (int)b->wide_chains; ++w)
+            if ((e = tc_launch_grouped(b->prec, b->chunked, w == 1, nullptr, 0, 0, nullptr, b->st)) != cudaSuccess)
+                return bail(cuda_fail(e, "grouped GEMM set-up"));
         if (start > 0x7fffffff / 256) return bail(fail(GAO_EINVAL, "batch GEMM has too many tiles"));
         b->tiles_per_suite = (int)start;
         // problem table order: largest GEMM first, so that the launch's tail is made of

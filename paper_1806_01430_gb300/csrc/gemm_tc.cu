@@ -60,7 +60,8 @@ constexpr int BM = 128;  // UMMA M (one TMEM lane per output row)
 constexpr int BK = 64;   // 64 bfloat16 = 128 bytes = one swizzle row
 constexpr int BK8 = 128; // 128 e4m3 = 128 bytes = one swizzle row
 constexpr int kMaxEpiWarps = 16;
-constexpr int kMaxSmemProblems = 448;  // grouped launch: problem starts kept in shared memory
+// grouped launch: problem starts kept in shared memory, next to the staging of eight or sixteen epilogue warps
+constexpr int max_smem_problems(int epi_warps) { return epi_warps > 8 ? 448 : 512; }
 constexpr int threads_tc(int epi_warps) { return 64 + 32 * epi_warps; }
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
 constexpr unsigned long long kDrainLimitNs = 200000000ull;  // 0.2 s
@@ -1092,8 +1093,9 @@ __global__ void __launch_bounds__(threads_tc(EW), 1)
     // every role looks up its tile's problem by binary search over the problems' first
     // tiles: keep them in shared memory (the persistent body synchronises the block
     // before any lookup)
-    __shared__ int s_starts[kMaxSmemProblems];
-    const bool in_smem = nprob <= kMaxSmemProblems;
+    constexpr int kMost = max_smem_problems(EW);
+    __shared__ int s_starts[kMost];
+    const bool in_smem = nprob <= kMost;
     if (in_smem)
         for (int i = threadIdx.x; i < nprob; i += blockDim.x) s_starts[i] = probs[i].tile_start;
     const ProblemTable src{probs, nprob, BN, in_smem ? s_starts : nullptr};
@@ -1695,11 +1697,6 @@ cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const floa
 // to hide it (4096^3 185 -> 162).  Elsewhere eight: the MMAs hide the rest, and sixteen warps'
 // 112 registers a thread cost 1 to 2% (4096^3 aligned, two or three terms, chain or not).
 int epi_warps(bool vec, bool fuse, int planes) { return !vec || (fuse && planes == 1) ? 16 : 8; }
-// ... of a grouped launch, whose problems' rows are of any alignment: sixteen where some problem
-// carries a chain and the products are few (the 16-program suite, three products: 180 us against
-// 196; six products: 283 against 265; without chains 148 against 134).
-int grouped_epi_warps(int prec, bool chain) { return chain && prec != GAO_GEMM_BF16X6 && prec != GAO_GEMM_FP8 ? 16 : 8; }
-
 }  // namespace
 
 // FP8 scratch: q(A) [Mp][Kp], q(B^T) [Np][Kp], then the scale-factor blocks of A
@@ -2201,7 +2198,7 @@ void tc_attach_chain(int prec, int64_t M, int64_t N, int64_t K, void* scratch, c
     prob->ep.fuse = 1;
 }
 
-cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* scratch, const TcFuse& fuse,
+cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* scratch, const TcFuse& fuse, bool wide,
                               cudaStream_t st, int* launches) {
     *launches = 0;
     if (M <= 0 || N <= 0) return cudaSuccess;
@@ -2209,7 +2206,7 @@ cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* s
     float* rpart = reinterpret_cast<float*>(reinterpret_cast<char*>(fpart) + tc_frob_partials_bytes(M, N));
     if (fuse.frob_out) {
         const int64_t tiles = (ru(M, BM) / BM) * ((N + 127) / 128);  // 128 x 128 tiles of the grouped launch
-        frob_partials_kernel<<<kFrobCtas, 128, 0, st>>>(fpart, tiles * grouped_epi_warps(prec, true), fuse.frob_out);
+        frob_partials_kernel<<<kFrobCtas, 128, 0, st>>>(fpart, tiles * (wide ? 16 : 8), fuse.frob_out);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         *launches += 1;
@@ -2224,24 +2221,26 @@ cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* s
     return cudaSuccess;
 }
 
-cudaError_t tc_launch_grouped(int prec, bool chunked, bool chain, const TcProblem* d_probs, int nprob, int total_tiles,
+bool tc_grouped_wide(int prec, int64_t tiles, int64_t unaligned) {
+    return prec == GAO_GEMM_BF16X3 && 6 * unaligned >= 5 * tiles;
+}
+
+cudaError_t tc_launch_grouped(int prec, bool chunked, bool wide, const TcProblem* d_probs, int nprob, int total_tiles,
                               int* err, cudaStream_t st) {
     // nprob == 0 / total_tiles == 0: only sets the kernel's shared-memory attribute
-    const bool wide = grouped_epi_warps(prec, chain) == 16;
+    if (wide) {
+        if (prec != GAO_GEMM_BF16X3) return cudaErrorInvalidValue;
+        return chunked ? launch_grouped_t<16, 128, 2, 3, 3, true>(d_probs, nprob, total_tiles, err, st)
+                       : launch_grouped_t<16, 128, 2, 3, 3, false>(d_probs, nprob, total_tiles, err, st);
+    }
     switch (prec) {
         case GAO_GEMM_BF16X6:
             return chunked ? launch_grouped_t<8, 128, 3, 6, 2, true>(d_probs, nprob, total_tiles, err, st)
                            : launch_grouped_t<8, 128, 3, 6, 2, false>(d_probs, nprob, total_tiles, err, st);
         case GAO_GEMM_BF16X3:
-            if (wide)
-                return chunked ? launch_grouped_t<16, 128, 2, 3, 3, true>(d_probs, nprob, total_tiles, err, st)
-                               : launch_grouped_t<16, 128, 2, 3, 3, false>(d_probs, nprob, total_tiles, err, st);
             return chunked ? launch_grouped_t<8, 128, 2, 3, 3, true>(d_probs, nprob, total_tiles, err, st)
                            : launch_grouped_t<8, 128, 2, 3, 3, false>(d_probs, nprob, total_tiles, err, st);
         case GAO_GEMM_BF16:
-            if (wide)
-                return chunked ? launch_grouped_t<16, 128, 1, 1, 6, true>(d_probs, nprob, total_tiles, err, st)
-                               : launch_grouped_t<16, 128, 1, 1, 6, false>(d_probs, nprob, total_tiles, err, st);
             return chunked ? launch_grouped_t<8, 128, 1, 1, 6, true>(d_probs, nprob, total_tiles, err, st)
                            : launch_grouped_t<8, 128, 1, 1, 6, false>(d_probs, nprob, total_tiles, err, st);
         case GAO_GEMM_FP8:

@@ -95,15 +95,25 @@ void tc_attach_chain(int prec, int64_t M, int64_t N, int64_t K, void* scratch, c
 
 // After a grouped launch with a fused chain: the norm from the per-warp partials and the
 // row sums from the block values of one problem (kernels on st).
-cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* scratch, const TcFuse& fuse,
+cudaError_t tc_finalize_chain(int prec, int64_t M, int64_t N, int64_t K, void* scratch, const TcFuse& fuse, bool wide,
                               cudaStream_t st, int* launches);
+
+// Whether the problems with a chain of a suite with so many tiles, `unaligned` of them of results
+// whose rows are not 16-byte aligned, run with sixteen epilogue warps (wide) rather than eight.
+// Settled by the suite, and the problems without a chain in a launch of their own, so that a
+// gene's kernel, and with it its time, does not depend on the genes it is measured beside.  Two
+// terms, 16 programs of 128 to 2048 rows, one gene and four in a launch, us, eight / sixteen warps:
+// 97 % of the tiles unaligned 195 / 186 and 794 / 687, 87 % 194 / 184 and 770 / 678; 78 % 178 / 183
+// and 725 / 682, 59 % 170 / 178 and 675 / 650; a single product gains at most 2 % at any share,
+// three terms lose 7 %, problems without a chain 10 %.
+bool tc_grouped_wide(int prec, int64_t tiles, int64_t unaligned);
 
 // One launch over nprob problems whose table (tile_start set, in order) is at d_probs
 // in device memory; every problem must come from tc_prepare with the same prec and
 // the same chunked-ness.  total_tiles = sum of tiles_m * tiles_n.  With total_tiles
-// = 0 it only prepares the kernel (shared-memory attribute), launching nothing.  chain: some
-// problem of the launch carries a chain (tc_attach_chain); each that does needs it set.
-cudaError_t tc_launch_grouped(int prec, bool chunked, bool chain, const TcProblem* d_probs, int nprob, int total_tiles,
+// = 0 it only prepares the kernel (shared-memory attribute), launching nothing.  wide: sixteen
+// epilogue warps.
+cudaError_t tc_launch_grouped(int prec, bool chunked, bool wide, const TcProblem* d_probs, int nprob, int total_tiles,
                               int* err, cudaStream_t st);
 
 }  // namespace gao
