@@ -14,7 +14,8 @@
 // lanes), with 8 x 16 three quarters of them.  Packed multiply-adds (fma.rn.f32x2: two columns
 // of a row, the same rounding per element) leave the issue slots that the loads, the operand
 // duplication and the loop need.  Both operands go to shared memory by cp.async (no register
-// staging): A as rows of BK elements (a thread reads four k of a row at once), B as it lies.
+// staging): A as rows of BK elements (a thread reads four k of a row at once), B as it lies; on the
+// large tiles, where rows are not 16-byte aligned, through registers (RAG).
 // A small problem has too few tiles to fill the GPU; since the chunks are summed apart anyway, a
 // cluster can split them (no order changes), and smaller tiles serve where that is not enough.
 // Measured, n x n x n, us (before: 128 x 128 tiles of 8 x 8 per thread, scalar FFMAs):
@@ -76,7 +77,12 @@ __device__ __forceinline__ void cp_async(uint32_t dst, const float* src, bool in
 // va, vb, vc: rows of A; of B; of C and C0 are 16-byte aligned.  SPLIT: a cluster of
 // ceil(K / kc) blocks along z shares a tile, each summing one chunk; the sums meet in shared
 // memory and each block adds, in chunk order, and stores its share of the tile.
-template <class S, bool SPLIT>
+// RAG: both operands go through registers, a word at a time and a step ahead, where cp.async would
+// move a word an instruction and lane: that cost the large tiles more than their loads' latency
+// (INIT and GEMM, us, cp.async -> registers: 2049^3 532 -> 483, 3001^3 1474 -> 1405, 8001 x 801 x 601
+// 257 -> 241; 256 threads of 8 x 8 before: 498, 1419, 259; only K of a few steps is better off with
+// cp.async, 5000 x 5000 x 33 120 -> 128, before 163).
+template <class S, bool SPLIT, bool RAG>
 __global__ void __launch_bounds__(S::THREADS, S::MINB)
     sgemm_kernel(float* C, const float* __restrict__ A, const float* __restrict__ B, const float* C0, int64_t M,
                  int64_t N, int64_t K, float alpha, float beta, int64_t kc, bool va, bool vb, bool vc) {
@@ -132,6 +138,29 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB)
         }
     };
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    constexpr int RA = RAG ? S::BM * BK / THREADS : 1, RB = RAG ? BK * S::BN / THREADS : 1;
+    float ra[RA], rb[RB];
+    auto fetch = [&](int64_t kt) {
+        const int64_t k0 = kbeg + kt * BK;
+#pragma unroll
+        for (int i = 0; i < RA; ++i) {
+            const int e = i * THREADS + t, r = e / BK, c = e % BK;
+            ra[i] = m0 + r < M && k0 + c < kend ? __ldg(A + (m0 + r) * K + k0 + c) : 0.0f;
+        }
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            const int e = i * THREADS + t, r = e / S::BN, c = e % S::BN;
+            rb[i] = k0 + r < kend && n0 + c < N ? __ldg(B + (k0 + r) * N + n0 + c) : 0.0f;
+        }
+    };
+    auto put = [&](int64_t kt) {
+        float* as = As + (int)(kt % S::STAGES) * S::A_FLOATS;
+        float* bs = Bs + (int)(kt % S::STAGES) * S::B_FLOATS;
+#pragma unroll
+        for (int i = 0; i < RA; ++i) as[(i * THREADS + t) / BK * S::LDA + (i * THREADS + t) % BK] = ra[i];
+#pragma unroll
+        for (int i = 0; i < RB; ++i) bs[i * THREADS + t] = rb[i];
+    };
 
     f32x2 acc[TM][TN / 2];
 #pragma unroll
@@ -148,18 +177,29 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB)
         for (int e = 0; e < S::E; ++e) ssum[e * THREADS + t] = make_float4(0, 0, 0, 0);
     }
 
+    if constexpr (RAG) {
+        if (nk > 0) {
+            fetch(0);
+            put(0);
+        }
+    } else {
 #pragma unroll
-    for (int s = 0; s < S::STAGES - 1; ++s) {
-        if (s < nk) load(s);
-        commit();
+        for (int s = 0; s < S::STAGES - 1; ++s) {
+            if (s < nk) load(s);
+            commit();
+        }
     }
     const int64_t chunk_tiles16 = kc / 16;  // 16-element steps per chunk
     int64_t left = chunk_tiles16;
     for (int64_t kt = 0; kt < nk; ++kt) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(S::STAGES - 2) : "memory");
+        if constexpr (!RAG) asm volatile("cp.async.wait_group %0;" ::"n"(S::STAGES - 2) : "memory");
         __syncthreads();  // stage kt has landed for every thread; everyone is done with stage kt - 1
-        if (kt + S::STAGES - 1 < nk) load(kt + S::STAGES - 1);
-        commit();
+        if constexpr (RAG) {
+            if (kt + 1 < nk) fetch(kt + 1);
+        } else {
+            if (kt + S::STAGES - 1 < nk) load(kt + S::STAGES - 1);
+            commit();
+        }
         const int st = (int)(kt % S::STAGES);
         const float* as = As + st * S::A_FLOATS + (wm * 4 * TM + ty) * S::LDA;  // rows ty, ty + 4, ...
         const float* bs = Bs + st * S::B_FLOATS + wn * 8 * TN + tx * 4;         // column quads 32 apart
@@ -214,6 +254,9 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB)
                         }
                 }
             }
+        }
+        if constexpr (RAG) {
+            if (kt + 1 < nk) put(kt + 1);  // its stage was last read before this step's barrier
         }
     }
 
@@ -291,10 +334,10 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB)
     }
 }
 
-template <class S, bool SPLIT>
+template <class S, bool SPLIT, bool RAG>
 cudaError_t launch_shape(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N, int64_t K,
                          float alpha, float beta, int64_t kc, cudaStream_t st) {
-    auto kern = sgemm_kernel<S, SPLIT>;
+    auto kern = sgemm_kernel<S, SPLIT, RAG>;
     constexpr int most = (int)(S::TILE_BYTES + S::SUM_BYTES);
     static bool attr_set = false;  // per instantiation
     if (!attr_set) {
@@ -331,7 +374,7 @@ cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const flo
     // estimated time: the fullest SM holds u blocks, which take max(lat, u w) clocks per element
     // of K (lat: a block alone, bound by latency; w: its share of a busy SM), plus a fixed cost
     // (launch, first loads, a split's exchange).  The figures are fits to times measured over
-    // n = 128 .. 4096 (within 10 %); rows that cp.async takes a word at a time cost `ragged` more.
+    // n = 128 .. 4096 (within 10 %); rows that are not 16-byte aligned cost `ragged` more.
     struct Model {
         int tile;
         double lat, w, fixed, fixed_split, ragged;
@@ -357,14 +400,14 @@ cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const flo
             best = i;
         }
     }
-#define GAO_SIMT(S, SPLIT) launch_shape<S, SPLIT>(C, A, B, C0, M, N, K, alpha, beta, kc, st)
+#define GAO_SIMT(S, SPLIT, RAG) launch_shape<S, SPLIT, RAG>(C, A, B, C0, M, N, K, alpha, beta, kc, st)
     switch (best) {
-        case 0: return GAO_SIMT(Large, false);
-        case 1: return GAO_SIMT(Large, true);
-        case 2: return GAO_SIMT(Medium, false);
-        case 3: return GAO_SIMT(Medium, true);
-        case 4: return GAO_SIMT(Small, false);
-        default: return GAO_SIMT(Small, true);
+        case 0: return rows16 ? GAO_SIMT(Large, false, false) : GAO_SIMT(Large, false, true);
+        case 1: return rows16 ? GAO_SIMT(Large, true, false) : GAO_SIMT(Large, true, true);
+        case 2: return GAO_SIMT(Medium, false, false);
+        case 3: return GAO_SIMT(Medium, true, false);
+        case 4: return GAO_SIMT(Small, false, false);
+        default: return GAO_SIMT(Small, true, false);
     }
 #undef GAO_SIMT
 }
