@@ -243,11 +243,13 @@ __global__ void __launch_bounds__(kThreads) host_copies_kernel(const __grid_cons
 // separate loop's operation, and written only where `out` is set.
 //
 // HBM-bound where its loads are in flight together.  A chain that reads one or two arrays (EXT)
-// loads kAhead quads (kAhead rows' quads in the reducing pass) of each before its first operation,
-// which then picks its operands from registers: fetching an operand when its operation comes
-// makes every operation of the chain wait for memory in turn, and reads an array again each
-// time it is named (the twelve-loop program's four loops on 6000 x 6000 with the last value written: 71.0 -> 64.6 us,
-// 432 MB).
+// loads them before its first operation (kAhead rows of them in the reducing pass), which then
+// picks its operands from registers: fetching an operand when its operation comes makes every
+// operation of the chain wait for memory in turn, and reads an array again each time it is named.
+// That gains where one value is written (INIT and chain, us: the twelve-loop program's four loops
+// 127.7 -> 119.4 on 6000 x 6000, 213.6 -> 200.7 on 8000 x 8000) and loses where the stores of two or
+// three bound the pass (8000 x 8000, two 240.7 -> 246.8, three of five loops 281 -> 289; four 328 ->
+// 332; five, two of them over earlier ones, 320 -> 340), so those fetch as they go.
 
 // One operation on N groups of four values: cur = op(x, y), x and y each the previous value or a
 // preloaded array's (EXT), or fetched by `fetch` now.  The branches are uniform: choosing by
@@ -318,31 +320,22 @@ __device__ __forceinline__ void chain_op(const EwChainOp& op, float (&cur)[N][4]
 
 template <bool EXT>
 __global__ void __launch_bounds__(256) ew_chain_kernel(const __grid_constant__ EwChain c) {
-    constexpr int kAhead = EXT ? 2 : 1;  // quads of a thread in flight
     const int64_t n = c.n;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
-    for (int64_t i0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i0 < n; i0 += kAhead * stride) {
-        float cur[kAhead][4] = {};
-        int w[kAhead];  // elements of each quad inside the array (a ragged last one element by element)
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
+        float cur[1][4] = {};
+        const bool vec = c.vec != 0 && i + 4 <= n;  // a ragged last quadruple element by element
+        const int w = n - i < 4 ? (int)(n - i) : 4;
+        auto fetch = [&](const float* src, float (&d)[1][4]) {
+            if (vec) {
+                const float4 v = *reinterpret_cast<const float4*>(src + i);
+                d[0][0] = v.x, d[0][1] = v.y, d[0][2] = v.z, d[0][3] = v.w;
+            } else {
 #pragma unroll
-        for (int k = 0; k < kAhead; ++k) {
-            const int64_t rest = n - (i0 + k * stride);
-            w[k] = rest >= 4 ? 4 : rest > 0 ? (int)rest : 0;
-        }
-        auto fetch = [&](const float* src, float (&d)[kAhead][4]) {
-#pragma unroll
-            for (int k = 0; k < kAhead; ++k) {
-                const float* p = src + i0 + k * stride;
-                if (c.vec && w[k] == 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(p);
-                    d[k][0] = v.x, d[k][1] = v.y, d[k][2] = v.z, d[k][3] = v.w;
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) d[k][q] = q < w[k] ? p[q] : 0.0f;
-                }
+                for (int q = 0; q < 4; ++q) d[0][q] = q < w ? src[i + q] : 0.0f;
             }
         };
-        float e0[kAhead][4], e1[kAhead][4];
+        float e0[1][4], e1[1][4];
         if constexpr (EXT) {
             fetch(c.ext[0], e0);
             if (c.next > 1) fetch(c.ext[1], e1);
@@ -350,18 +343,14 @@ __global__ void __launch_bounds__(256) ew_chain_kernel(const __grid_constant__ E
 #pragma unroll 1
         for (int o = 0; o < c.nops; ++o) {
             const EwChainOp& op = c.op[o];
-            chain_op<EXT, kAhead>(op, cur, e0, e1, fetch);
+            chain_op<EXT, 1>(op, cur, e0, e1, fetch);
             if (op.out) {
+                if (vec) {
+                    *reinterpret_cast<float4*>(op.out + i) = make_float4(cur[0][0], cur[0][1], cur[0][2], cur[0][3]);
+                } else {
 #pragma unroll
-                for (int k = 0; k < kAhead; ++k) {
-                    float* p = op.out + i0 + k * stride;
-                    if (c.vec && w[k] == 4) {
-                        *reinterpret_cast<float4*>(p) = make_float4(cur[k][0], cur[k][1], cur[k][2], cur[k][3]);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (q < w[k]) p[q] = cur[k][q];
-                    }
+                    for (int q = 0; q < 4; ++q)
+                        if (q < w) op.out[i + q] = cur[0][q];
                 }
             }
         }
@@ -1403,7 +1392,9 @@ cudaError_t launch_ew_chain(const EwChain& c, cudaStream_t st) {
     if (c.n <= 0) return cudaSuccess;
     EwChain k = c;
     k.vec = chain_fields(k);
-    if (k.next > 0) ew_chain_kernel<true><<<grid_for((c.n + 7) / 8), kThreads, 0, st>>>(k);
+    int written = 0;
+    for (int o = 0; o < c.nops; ++o) written += c.op[o].out != nullptr;
+    if (k.next > 0 && written == 1) ew_chain_kernel<true><<<grid_for((c.n + 3) / 4), kThreads, 0, st>>>(k);
     else ew_chain_kernel<false><<<grid_for((c.n + 3) / 4), kThreads, 0, st>>>(k);
     return cudaGetLastError();
 }
