@@ -221,7 +221,7 @@ cudaError_t launch_edge_chain(const float* in, float* bout, int64_t rows, int64_
                               float alpha, bool swap, float* g1, float* g2, float* s1, float* s2, float* m,
                               cudaStream_t st, int64_t row_begin = 0, int64_t row_end = -1,
                               const GradReduce* red = nullptr, int* launches = nullptr);
-int64_t edge_chain_blocks(int64_t rows, int64_t cols);
+int64_t edge_chain_blocks(int64_t rows, int64_t cols, bool stores);  // stores: some per-pixel output is written
 int64_t edge_chain_blocks_max(int64_t cols);
 
 // Weights of the 3x3 stencil presets of GAO_LOOP_STENCIL3, row-major over (a, b).

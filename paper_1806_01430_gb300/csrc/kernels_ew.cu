@@ -1024,7 +1024,10 @@ __global__ void __launch_bounds__(kStencilThreads, CHAIN ? kChainBlocks : 8)
 // 8192 x 8192: 84 us; 107 with a column an instruction, moves and a second, part-filled wave.
 constexpr int kEdgeNC = 8;               // columns a lane holds
 constexpr int kEdgeCols = 30 * kEdgeNC;  // output columns of a warp (lanes 1 .. 30)
-constexpr int kEdgeBlocks = 4;           // resident 128-thread blocks per SM the kernel is built for
+// Resident 128-thread blocks per SM the kernel is built for.  Where it stores per-pixel values, 168
+// registers a thread and not 128, which spill (INIT and pass, us: 2160 x 3840 with its magnitude
+// written 47.6 -> 43.7, 4096 x 4096 66.5 -> 61.7).
+constexpr int edge_blocks(bool stores) { return stores ? 3 : 4; }
 constexpr int kEdgeBlockCols = kEdgeCols * (kStencilThreads / 32);  // output columns of a block
 
 using f32x2 = unsigned long long;  // two binary32 values, the first in the low half
@@ -1064,21 +1067,34 @@ struct EdgeRow {
     float4 g[2];
 };
 
+// Which of a lane's eight columns: the first n (with 16-byte rows none, four or eight: two flags that
+// stay in predicates; else a count, where eight flags would not).
+struct EdgeCols {
+    int n;
+    bool lo, hi;
+    __device__ __forceinline__ explicit EdgeCols(int count) : n(count), lo(count > 0), hi(count > 4) {}
+    template <bool VEC>
+    __device__ __forceinline__ bool has(int q) const {
+        return VEC ? (q < 4 ? lo : hi) : q < n;
+    }
+};
+
 // p: row y's first column of the lane (any value when the row is outside the image).
 template <bool VEC>
-__device__ __forceinline__ void edge_load(EdgeRow& r, const float* __restrict__ p, bool row_in, const bool inc[kEdgeNC]) {
+__device__ __forceinline__ void edge_load(EdgeRow& r, const float* __restrict__ p, bool row_in,
+                                          const EdgeCols& in) {
     r.g[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     r.g[1] = r.g[0];
     if (!row_in) return;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         if (VEC) {
-            if (inc[4 * k]) r.g[k] = __ldg(reinterpret_cast<const float4*>(p + 4 * k));
+            if (in.has<VEC>(4 * k)) r.g[k] = __ldg(reinterpret_cast<const float4*>(p + 4 * k));
         } else {
-            if (inc[4 * k]) r.g[k].x = __ldg(p + 4 * k);
-            if (inc[4 * k + 1]) r.g[k].y = __ldg(p + 4 * k + 1);
-            if (inc[4 * k + 2]) r.g[k].z = __ldg(p + 4 * k + 2);
-            if (inc[4 * k + 3]) r.g[k].w = __ldg(p + 4 * k + 3);
+            if (in.has<VEC>(4 * k)) r.g[k].x = __ldg(p + 4 * k);
+            if (in.has<VEC>(4 * k + 1)) r.g[k].y = __ldg(p + 4 * k + 1);
+            if (in.has<VEC>(4 * k + 2)) r.g[k].z = __ldg(p + 4 * k + 2);
+            if (in.has<VEC>(4 * k + 3)) r.g[k].w = __ldg(p + 4 * k + 3);
         }
     }
 }
@@ -1099,8 +1115,13 @@ __device__ __forceinline__ void edge_pairs(EdgePairs& r, const EdgeRow& v) {
     edge_spread(r);
 }
 
+// A row's produced columns stored (every lane of the warp takes part): with 16-byte rows straight
+// from the lanes, else through the warp's 256 words of shared memory, so that each store covers
+// 32 consecutive columns and not a word every 32 bytes (pass, us: 4095 x 4097 with its magnitude
+// written 109 -> 70, 2000 x 2001 with three of its maps 81.5 -> 36.4).
 template <bool VEC>
-__device__ __forceinline__ void edge_store(float* row, int64_t c0, const bool outc[kEdgeNC], const f32x2 v[4]) {
+__device__ __forceinline__ void edge_store(float* row, int64_t c0, int64_t cols, const EdgeCols& out, const f32x2 v[4],
+                                           float* stage) {
     float x[kEdgeNC];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -1108,15 +1129,26 @@ __device__ __forceinline__ void edge_store(float* row, int64_t c0, const bool ou
         x[k] = u.x;
         x[k + 4] = u.y;
     }
+    if (VEC) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        if (VEC) {
-            if (outc[4 * k])
+        for (int k = 0; k < 2; ++k)
+            if (out.has<VEC>(4 * k))
                 *reinterpret_cast<float4*>(row + c0 + 4 * k) = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
-        } else {
+    } else {
+        const int lane = threadIdx.x & 31;
+        __syncwarp();  // the previous row's reads are done
 #pragma unroll
-            for (int q = 4 * k; q < 4 * k + 4; ++q)
-                if (outc[q]) row[c0 + q] = x[q];
+        for (int k = 0; k < 2; ++k)
+            *reinterpret_cast<float4*>(stage + kEdgeNC * lane + 4 * k) =
+                make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+        __syncwarp();
+        const int64_t cw = c0 - kEdgeNC * lane;  // the warp's first column
+        const int end = cols - cw < 31 * kEdgeNC ? (int)(cols - cw) : 31 * kEdgeNC;
+        float* p = row + cw + lane;
+#pragma unroll
+        for (int k = 0; k < kEdgeNC; ++k) {
+            const int i = 32 * k + lane;
+            if (i >= kEdgeNC && i < end) p[32 * k] = stage[i];
         }
     }
 }
@@ -1136,7 +1168,7 @@ __device__ __forceinline__ f32x2 stencil9_pair(const StencilW& w, const EdgePair
 }
 
 template <bool VEC, int P0, int P1, int P2, bool RED, bool STORE>
-__global__ void __launch_bounds__(kStencilThreads, kEdgeBlocks)
+__global__ void __launch_bounds__(kStencilThreads, edge_blocks(STORE))
     edge_chain_kernel(StencilOut out, float* __restrict__ bout, const float* __restrict__ in, int64_t rows,
                       int64_t cols, StencilW w0, StencilW w1, StencilW w2, int strip, int64_t row_begin,
                       int64_t row_end) {
@@ -1146,23 +1178,20 @@ __global__ void __launch_bounds__(kStencilThreads, kEdgeBlocks)
 #pragma unroll
     for (int q = 0; q < NC; ++q) mk[q] = 0u;
     const int lane = threadIdx.x & 31;
+    constexpr int kStage = STORE && !VEC ? 32 * NC : 4;  // floats of a warp's staging row
+    __shared__ __align__(16) float s_stage[kStencilThreads / 32][kStage];
+    float* stage = s_stage[threadIdx.x >> 5];
     const int64_t c0 = ((int64_t)blockIdx.x * (kStencilThreads / 32) + (threadIdx.x >> 5)) * kEdgeCols - NC + NC * lane;
-    bool inc[NC], outc[NC];  // column c0 + q inside the image; and produced by this lane
-#pragma unroll
-    for (int q = 0; q < NC; ++q) {
-        const int64_t c = VEC ? c0 + (q & ~3) : c0 + q;  // with 16-byte rows, by groups of four
-        inc[q] = c >= 0 && c < cols;
-        outc[q] = inc[q] && lane >= 1 && lane <= 30;
-    }
+    // this lane's columns inside the image, and those it produces
+    const EdgeCols inc(c0 < 0 || c0 >= cols ? 0 : cols - c0 < NC ? (int)(cols - c0) : NC);
+    const EdgeCols outc(lane >= 1 && lane <= 30 ? inc.n : 0);
     // output rows [r0, r1) of this block's strip; raw rows r0 - 2 .. r1 + 1 are read
     const int64_t r0 = row_begin + (int64_t)blockIdx.y * strip;
     const int64_t r1 = r0 + strip < row_end ? r0 + strip : row_end;
     const int64_t ylim = r1 + 2 < rows ? r1 + 2 : rows;
     // a lane whose columns are all inside the image zeroes none of its B values but in the
     // rows above and below it, so it skips the per-value choice elsewhere
-    bool all_in = true;
-#pragma unroll
-    for (int q = 0; q < NC; ++q) all_in = all_in && inc[q];
+    const bool all_in = inc.n == NC;
     // B's row from the raw rows above, at and below it (zero outside the image)
     auto blur = [&](EdgePairs& b, const EdgePairs& xu, const EdgePairs& xm, const EdgePairs& xd, bool row_in) {
 #pragma unroll
@@ -1171,12 +1200,12 @@ __global__ void __launch_bounds__(kStencilThreads, kEdgeBlocks)
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float2 u = unpack2(b.p[k + 1]);
-                b.p[k + 1] = pack2(row_in && inc[k] ? u.x : 0.0f, row_in && inc[k + 4] ? u.y : 0.0f);
+                b.p[k + 1] = pack2(row_in && inc.has<VEC>(k) ? u.x : 0.0f, row_in && inc.has<VEC>(k + 4) ? u.y : 0.0f);
             }
         }
     };
     auto store_b = [&](int64_t y, const EdgePairs& b) {
-        if (STORE && bout && y >= r0 && y < r1) edge_store<VEC>(bout + y * cols, c0, outc, b.p + 1);
+        if (STORE && bout && y >= r0 && y < r1) edge_store<VEC>(bout + y * cols, c0, cols, outc, b.p + 1, stage);
     };
     auto row_ptr = [&](int64_t y) { return in + y * cols + c0; };
     auto load_row = [&](EdgeRow& v, int64_t y) { edge_load<VEC>(v, row_ptr(y), y >= 0 && y < ylim, inc); };
@@ -1224,11 +1253,11 @@ __global__ void __launch_bounds__(kStencilThreads, kEdgeBlocks)
         }
         if constexpr (STORE) {
             const int64_t off = row * cols;
-            if (out.g1) edge_store<VEC>(out.g1 + off, c0, outc, o);
-            if (out.g2) edge_store<VEC>(out.g2 + off, c0, outc, o2);
-            if (out.s1) edge_store<VEC>(out.s1 + off, c0, outc, a);
-            if (out.s2) edge_store<VEC>(out.s2 + off, c0, outc, b);
-            if (out.m) edge_store<VEC>(out.m + off, c0, outc, m);  // null when only the reductions read m
+            if (out.g1) edge_store<VEC>(out.g1 + off, c0, cols, outc, o, stage);
+            if (out.g2) edge_store<VEC>(out.g2 + off, c0, cols, outc, o2, stage);
+            if (out.s1) edge_store<VEC>(out.s1 + off, c0, cols, outc, a, stage);
+            if (out.s2) edge_store<VEC>(out.s2 + off, c0, cols, outc, b, stage);
+            if (out.m) edge_store<VEC>(out.m + off, c0, cols, outc, m, stage);  // null when only the reductions read m
         }
         if constexpr (RED) {
             // the keys of every column are kept and only those of produced columns are raised at
@@ -1249,10 +1278,10 @@ __global__ void __launch_bounds__(kStencilThreads, kEdgeBlocks)
                 float t;
                 if (VEC) {
                     const float2 g = unpack2(add2(add2(m[0], m[1]), add2(m[2], m[3])));
-                    t = g.x + (inc[4] ? g.y : 0.0f);
+                    t = g.x + (inc.hi ? g.y : 0.0f);
                 } else {
 #pragma unroll
-                    for (int q = 0; q < NC; ++q) v[q] = outc[q] ? v[q] : 0.0f;
+                    for (int q = 0; q < NC; ++q) v[q] = outc.has<VEC>(q) ? v[q] : 0.0f;
                     t = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
                 }
                 comp_add(rs, rc, t);
@@ -1270,11 +1299,11 @@ __global__ void __launch_bounds__(kStencilThreads, kEdgeBlocks)
         if (out.keys && r1 > r0) {
 #pragma unroll
             for (int q = 0; q < NC; ++q)
-                if (outc[q]) atomicMax(out.keys + c0 + q, mk[q]);  // max: exact and order-free
+                if (outc.has<VEC>(q)) atomicMax(out.keys + c0 + q, mk[q]);  // max: exact and order-free
         }
         if (out.part) {
             __shared__ double wsum[kStencilThreads / 32];
-            double acc = (!VEC || outc[0]) ? (double)rs + (double)rc : 0.0;
+            double acc = (!VEC || outc.lo) ? (double)rs + (double)rc : 0.0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (lane == 0) wsum[threadIdx.x >> 5] = acc;
@@ -1664,10 +1693,12 @@ namespace {
 // strips of rows for one wave of the resident blocks (each strip reads four raw rows beyond its
 // own and blurs two, so taller strips repeat less; a second wave would also start late), at
 // least 16 rows per strip.
-int64_t edge_strips(int64_t gx) { return std::max<int64_t>(1, (int64_t)sm_count() * kEdgeBlocks / gx); }
-void edge_grid(int64_t span, int64_t cols, int64_t* gx, int64_t* strip, int64_t* gy) {
+int64_t edge_strips(int64_t gx, bool stores) {
+    return std::max<int64_t>(1, (int64_t)sm_count() * edge_blocks(stores) / gx);
+}
+void edge_grid(int64_t span, int64_t cols, bool stores, int64_t* gx, int64_t* strip, int64_t* gy) {
     *gx = (cols + kEdgeBlockCols - 1) / kEdgeBlockCols;
-    const int64_t strips = edge_strips(*gx);
+    const int64_t strips = edge_strips(*gx, stores);
     int64_t s = (span + strips - 1) / strips;
     if (s < 16) s = 16;
     if ((span + s - 1) / s > 65535) s = (span + 65534) / 65535;
@@ -1676,10 +1707,10 @@ void edge_grid(int64_t span, int64_t cols, int64_t* gx, int64_t* strip, int64_t*
 }
 }  // namespace
 
-int64_t edge_chain_blocks(int64_t rows, int64_t cols) {
+int64_t edge_chain_blocks(int64_t rows, int64_t cols, bool stores) {
     if (rows <= 0 || cols <= 0) return 0;
     int64_t gx, strip, gy;
-    edge_grid(rows, cols, &gx, &strip, &gy);
+    edge_grid(rows, cols, stores, &gx, &strip, &gy);
     return gx * gy;
 }
 
@@ -1688,7 +1719,7 @@ int64_t edge_chain_blocks(int64_t rows, int64_t cols) {
 int64_t edge_chain_blocks_max(int64_t cols) {
     if (cols <= 0) return 0;
     const int64_t gx = (cols + kEdgeBlockCols - 1) / kEdgeBlockCols;
-    return gx * edge_strips(gx);
+    return gx * std::max(edge_strips(gx, false), edge_strips(gx, true));
 }
 
 cudaError_t launch_edge_chain(const float* in, float* bout, int64_t rows, int64_t cols, int p0, int p1, int p2,
@@ -1704,7 +1735,8 @@ cudaError_t launch_edge_chain(const float* in, float* bout, int64_t rows, int64_
         return cudaErrorInvalidValue;
     const bool want_sum = red && red->sum_out, want_max = red && red->colmax_out;
     const int64_t span = row_end - row_begin;
-    const int64_t nblk = edge_chain_blocks(span, cols);  // this launch's partials
+    const bool stores = bout || m || g1 || g2 || s1 || s2;  // per-pixel outputs (else reductions only)
+    const int64_t nblk = edge_chain_blocks(span, cols, stores);  // this launch's partials
     if (want_sum && (!red->part || red->part_at < 0 || red->part_cap < red->part_at + nblk)) return cudaErrorInvalidValue;
     if (want_max && !red->keys) return cudaErrorInvalidValue;
     const StencilOut o{g1, g2, s1, s2, m, alpha, swap ? 1 : 0, want_sum ? red->part + red->part_at : nullptr,
@@ -1715,14 +1747,13 @@ cudaError_t launch_edge_chain(const float* in, float* bout, int64_t rows, int64_
     }
     if (span > 0 && cols > 0) {
         int64_t gx, strip, gy;
-        edge_grid(span, cols, &gx, &strip, &gy);
+        edge_grid(span, cols, stores, &gx, &strip, &gy);
         if (gx > 0x7fffffff || strip > 0x7fffffff) return cudaErrorInvalidValue;
         const dim3 grid((unsigned)gx, (unsigned)gy);
         const uintptr_t ptrs = (uintptr_t)in | (uintptr_t)bout | (uintptr_t)m | (uintptr_t)g1 | (uintptr_t)g2 |
                                (uintptr_t)s1 | (uintptr_t)s2;
         const bool vec = (cols % 4 == 0) && (ptrs & 15u) == 0;
         const bool reduce = want_sum || want_max;
-        const bool stores = bout || m || g1 || g2 || s1 || s2;  // per-pixel outputs (else reductions only)
         const int sp = (int)strip;
 #define GAO_EDGE_LAUNCH(V, A, B, C, R, S)                                                                \
     edge_chain_kernel<V, A, B, C, R, S><<<grid, kStencilThreads, 0, st>>>(o, bout, in, rows, cols, w0, w1, w2, \

@@ -283,7 +283,8 @@ Layout plan(const gao_loop* loops, int n_loops, const gao_buffer* bufs, int n_bu
             // chain alone or with the blur before it
             const int64_t r = bufs[lp.ins[0]].rows, c = bufs[lp.ins[0]].cols;
             const int64_t blocks = std::max({grad_chain_blocks(r, c), kMaxRowBlocks * grad_chain_blocks_max(c),
-                                             edge_chain_blocks(r, c), kMaxRowBlocks * edge_chain_blocks_max(c)});
+                                             edge_chain_blocks(r, c, false), edge_chain_blocks(r, c, true),
+                                             kMaxRowBlocks * edge_chain_blocks_max(c)});
             chainpart = std::max(chainpart, (size_t)blocks * 8);
         }
         if (lp.kind == GAO_LOOP_INIT)
@@ -1579,7 +1580,7 @@ gao_status run_gpu_stencil_pipelined(RunCtx& R, int li, const GradChain* gch, bo
                                               reduce ? &red : nullptr, &nl);
             if (e != cudaSuccess) return cuda_fail(e, "blur and gradient chain strip launch");
             S.launches += nl;
-            red.part_at += edge_chain_blocks(f1 - formed, cols);
+            red.part_at += edge_chain_blocks(f1 - formed, cols, !written.empty());
             if ((sst = send_rows(formed, f1)) != GAO_OK) return sst;
             formed = f1;
         }
