@@ -663,8 +663,9 @@ struct TileInfo {
 };
 
 // Tiles of one problem (kernel arguments).
+template <bool ANY>
 struct OneProblem {
-    static constexpr bool kGrouped = false;
+    static constexpr bool kAnyRow = ANY;  // its rows may be of any alignment
     const CUtensorMap* ta;
     const CUtensorMap* tb;
     EpiArgs ep;
@@ -694,7 +695,7 @@ struct OneProblem {
 // Tiles of a grouped launch: tile t belongs to the problem whose range holds t
 // (binary search over tile_start, which increases along the table).
 struct ProblemTable {
-    static constexpr bool kGrouped = true;
+    static constexpr bool kAnyRow = true;
     const TcProblem* probs;
     int nprob, bn;
     const int* starts;  // shared-memory copy of every problem's tile_start (null: read probs)
@@ -963,7 +964,7 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         float* stg = stg_all + ew * (Stg<EW>::BYTES / 4);
         constexpr int G = kEpiCols / 32;  // 32-column groups per thread
-        constexpr bool ANYROW = EW > 8 || Src::kGrouped;  // eight warps in a launch of its own: see epi_warps
+        constexpr bool ANYROW = Src::kAnyRow;
         int gc = 0;
         bool ok = true;
         for (int t = first_tile; t < total_tiles && ok; t += tile_step) {
@@ -1065,12 +1066,12 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
     }
 }
 
-template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, int EW>
+template <int BN, int PA, int PB, int NPROD, int STAGES, bool CHUNKED, bool FP8, int EW, bool ANY>
 __global__ void __launch_bounds__(threads_tc(EW), 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiArgs ep,
                    int Mp, int Np, int num_kb, int chunk_kb, int tiles_m, int tiles_n, int group, int pf_kb,
                    int* err) {
-    const OneProblem src{&tmA, &tmB, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group, BN, pf_kb, BM};
+    const OneProblem<ANY> src{&tmA, &tmB, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group, BN, pf_kb, BM};
     gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, false, EW>(src, tiles_m * tiles_n, err);
 }
 
@@ -1082,7 +1083,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_tc(EW), 1)
                         const __grid_constant__ CUtensorMap tmSA, const __grid_constant__ CUtensorMap tmSB, EpiArgs ep,
                         int Mp, int Np, int num_kb, int chunk_kb, int tiles_m, int tiles_n, int group, int pf_kb,
                         int* err) {
-    const OneProblem src{&tmA,  &tmB, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group, BN, pf_kb, 2 * BM,
+    const OneProblem<(EW > 8)> src{&tmA,  &tmB, ep, Mp, Np, num_kb, chunk_kb, tiles_m, tiles_n, group, BN, pf_kb, 2 * BM,
                          &tmSA, &tmSB};
     gemm_tc_persistent<BN, PA, PB, NPROD, STAGES, CHUNKED, FP8, true, EW>(src, tiles_m * tiles_n, err);
 }
@@ -1624,12 +1625,12 @@ bool make_map(CUtensorMap* map, void* base, int64_t inner, int64_t rows, int box
     return true;
 }
 
-template <int EW, int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false>
+template <int EW, int BN, int P, int NPROD, int STAGES, bool CHUNKED, bool FP8 = false, bool ANY = (EW > 8)>
 cudaError_t launch_mma(const CUtensorMap& ta, const CUtensorMap& tb, const EpiArgs& ep, int Mp, int Np, int num_kb,
                        int chunk_kb, int group, int pf_kb, int* err, cudaStream_t st) {
     // Np is the plane stride (a multiple of 256); only ceil(N / BN) column tiles hold data
     using Cfg = TcCfg<BN, P, P, NPROD, STAGES, CHUNKED, FP8, false, EW>;
-    auto kern = gemm_tc_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8, EW>;
+    auto kern = gemm_tc_kernel<BN, P, P, NPROD, STAGES, CHUNKED, FP8, EW, ANY>;
     static bool attr_set = false;  // per instantiation
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
@@ -1692,11 +1693,21 @@ cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const floa
 
 // Epilogue warps of a launch.  An epilogue bound by the latency of its C0 / X loads and staging
 // round trips takes sixteen: rows that are not 16-byte aligned, a word a lane (GEMM with
-// 8 -> 16 warps, us: 4001 x 500 x 3003, two terms 82 -> 60; FP8 3000 x 4100 x 5003 100 -> 88; six-loop chain at
-// 4095, three terms 611 -> 573), and the chain behind a single product, whose MMAs are too few
+// 8 -> 16 warps, us: 4001 x 500 x 3003, two terms 82 -> 60; FP8 3000 x 4100 x 5003 100 -> 88; six-loop
+// chain at 4095, three terms 611 -> 573), and the chain behind a single product, whose MMAs are too few
 // to hide it (4096^3 185 -> 162).  Elsewhere eight: the MMAs hide the rest, and sixteen warps'
 // 112 registers a thread cost 1 to 2% (4096^3 aligned, two or three terms, chain or not).
-int epi_warps(bool vec, bool fuse, int planes) { return !vec || (fuse && planes == 1) ? 16 : 8; }
+// Unaligned rows without a chain are hidden too behind a long inner dimension and enough tiles
+// an SM t (M, N, K, us, eight / sixteen; two terms: 4097, 4095, 1501 139 / 138, 2050 173 / 175, 4100 303 /
+// 307, 6001, 6001, 1001 195 / 195, 1501 270 / 276; three: 4097, 4095, 2050 300 / 297, 3001 406 / 409, 4100
+// 546 / 554, 6001, 6001, 1501 453 / 449, 2050 604 / 616, 4100 1127 / 1159; 2001, 2001, 3001, where the last
+// round of tiles shows, 131 / 125).
+int epi_warps(bool vec, bool fuse, int planes, bool pair, int64_t M, int64_t N, int64_t K) {
+    if (vec) return fuse && planes == 1 ? 16 : 8;
+    if (fuse || pair || planes == 1) return 16;
+    const double t = (double)(((M + BM - 1) / BM) * ((N + 127) / 128)) / (double)sm_count();
+    return t >= 4.0 && ((double)K >= 1000.0 * planes || t * (double)K >= 8000.0 * planes) ? 8 : 16;
+}
 }  // namespace
 
 // FP8 scratch: q(A) [Mp][Kp], q(B^T) [Np][Kp], then the scale-factor blocks of A
@@ -1961,7 +1972,7 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
     float* rpart = reinterpret_cast<float*>(reinterpret_cast<char*>(fpart) + tc_frob_partials_bytes(Mlay, N));
     const int64_t tiles_n = (N + bn - 1) / bn;
     ep.ldE = M;
-    const int ew = epi_warps(ep.vec != 0, fuse != nullptr, P);
+    const int ew = epi_warps(ep.vec != 0, fuse != nullptr, P, pair, M, ncols, K);
     if (fuse) {
         ep.X = fuse->X;
         ep.D = fuse->D;
@@ -1993,7 +2004,16 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
              : chunked   ? launch_mma<EW, 128, 1, 1, 6, true>(GAO_TC_ARGS)                                            \
              : bn == 256 ? launch_mma<EW, 256, 1, 1, 4, false>(GAO_TC_ARGS)                                           \
                          : launch_mma<EW, 128, 1, 1, 6, false>(GAO_TC_ARGS)))
-    e = ew == 16 ? GAO_TC_LAUNCH(16) : GAO_TC_LAUNCH(8);
+    if (ew == 8 && !ep.vec) {  // two or three terms on one CTA, no chain
+        if (P == 3)
+            e = chunked ? launch_mma<8, 128, 3, 6, 2, true, false, true>(GAO_TC_ARGS)
+                        : launch_mma<8, 128, 3, 6, 2, false, false, true>(GAO_TC_ARGS);
+        else
+            e = chunked ? launch_mma<8, 128, 2, 3, 3, true, false, true>(GAO_TC_ARGS)
+                        : launch_mma<8, 128, 2, 3, 3, false, false, true>(GAO_TC_ARGS);
+    } else {
+        e = ew == 16 ? GAO_TC_LAUNCH(16) : GAO_TC_LAUNCH(8);
+    }
 #undef GAO_TC_LAUNCH
 #undef GAO_TC_ARGS
     if (e != cudaSuccess) return e;
@@ -2049,7 +2069,7 @@ cudaError_t launch_gemm_fp8(float* C, const float* A, const float* B, const floa
                reinterpret_cast<const float*>(sa), reinterpret_cast<const float*>(sb), (int)L.kbs, (int)L.Np};
     if (ev.k0) record_timing(ev.k0, st);
     const int kbs = (int)L.kbs;
-    const int ew = epi_warps(ep.vec != 0, false, 1);
+    const int ew = epi_warps(ep.vec != 0, false, 1, pair, M, N, K);
     cudaError_t e;
     if (pair) {
         CUtensorMap tsa, tsb;
