@@ -175,6 +175,12 @@ void gemm_shape(const gao_prog* p, int gl, int64_t* m, int64_t* nn, int64_t* k) 
     *nn = p->bufs[(size_t)L.ins[1]].d.cols;
 }
 
+double gemm_work(const gao_prog* p, int gl) {
+    int64_t m, n, k;
+    gemm_shape(p, gl, &m, &n, &k);
+    return (double)m * (double)n * (double)k;
+}
+
 // Capture the GPU work of loop li for every program of replica R into one graph.  For the
 // grouped GEMM loop the graph holds the operand splits only, and R.probs describes the
 // problems for the grouped launch made at run time.
@@ -192,6 +198,9 @@ gao_status capture_phase(gao_batch* b, Replica& R, int li) {
         order = b->gemm_order;
         R.probs.assign(R.progs.size(), TcProblem{});
     }
+    double total = 0.0;  // of the GEMMs that share the GPU
+    if (li == b->gemm_loop)
+        for (const gao_prog* p : R.progs) total += gemm_work(p, li);
     for (size_t j = 0; j < order.size() && e == cudaSuccess && status == GAO_OK && !group_init; ++j) {
         gao_prog* p = R.progs[order[j]];
         cudaStream_t s = b->side[j % kSide];
@@ -210,6 +219,7 @@ gao_status capture_phase(gao_batch* b, Replica& R, int li) {
             kernels += nl;
         } else {
             RunCtx rc{p, 0.0, false, CpuCtx{p->opts.cpu_threads, 0.0, false}, s, false};
+            if (li == b->gemm_loop) rc.beside = total / std::max(1.0, gemm_work(p, li));
             const int before = p->stats[(size_t)li].launches;
             status = run_gpu_loop(rc, li);
             kernels += p->stats[(size_t)li].launches - before;
@@ -766,10 +776,7 @@ extern "C" gao_status batch_create(gao_prog* const* progs, int n_progs, gao_batc
         b->gemm_order.resize((size_t)n_progs);
         std::iota(b->gemm_order.begin(), b->gemm_order.end(), 0);
         std::stable_sort(b->gemm_order.begin(), b->gemm_order.end(), [&](size_t x, size_t y) {
-            int64_t mx, nx, kx, my, ny, ky;
-            gemm_shape(progs[x], b->gemm_loop, &mx, &nx, &kx);
-            gemm_shape(progs[y], b->gemm_loop, &my, &ny, &ky);
-            return (double)mx * nx * kx > (double)my * ny * ky;
+            return gemm_work(progs[x], b->gemm_loop) > gemm_work(progs[y], b->gemm_loop);
         });
     }
     // the first INIT loop without row scaling: one grouped launch over every program's

@@ -247,9 +247,9 @@ inline bool stencil_weights(int preset, float w[9]) {
 cudaError_t launch_wait_selftest(int* flag, int* err, double limit_s, cudaStream_t st);
 
 // FP32 SIMT GEMM: C = alpha*A@B + beta*C0 (C may alias C0).  kchunk: K elements per
-// binary32 partial sum (<= 0: one sum over all of K).
+// binary32 partial sum (<= 0: one sum over all of K).  1 / beside: its part of the work on the GPU.
 cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N,
-                             int64_t K, float alpha, float beta, int kchunk, cudaStream_t st);
+                             int64_t K, float alpha, float beta, int kchunk, cudaStream_t st, double beside = 1.0);
 
 // Tensor-core GEMM (split operands + tcgen05).  Scratch layout and size are given
 // by tc_scratch_bytes; `err` receives DEV_* codes.

@@ -366,7 +366,7 @@ cudaError_t launch_shape(float* C, const float* A, const float* B, const float* 
 }  // namespace
 
 cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const float* C0, int64_t M, int64_t N,
-                             int64_t K, float alpha, float beta, int kchunk, cudaStream_t st) {
+                             int64_t K, float alpha, float beta, int kchunk, cudaStream_t st, double beside) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if ((M + 127) / 128 > 65535) return cudaErrorInvalidValue;
     const int64_t kc = kchunk > 0 ? (((int64_t)kchunk + 15) / 16) * 16 : (int64_t)1 << 40;  // above any K: one chunk
@@ -374,7 +374,10 @@ cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const flo
     // estimated time: the fullest SM holds u blocks, which take max(lat, u w) clocks per element
     // of K (lat: a block alone, bound by latency; w: its share of a busy SM), plus a fixed cost
     // (launch, first loads, a split's exchange).  The figures are fits to times measured over
-    // n = 128 .. 4096 (within 10 %); rows that are not 16-byte aligned cost `ragged` more.
+    // n = 128 .. 4096 (within 10 %); a GEMM that shares the GPU with others' is taken to have its
+    // part of the SMs, since the small tiles' extra loads then cost all of them (whole batches, us, as if
+    // alone / so / 128 x 128 tiles of 256 threads for all: 20 programs of 100 to 2000 rows, unaligned,
+    // 1930 / 1847 / 1790, aligned 1532 / 1519 / 1622; eight of 512 to 1024 494 / 428 / 475); rows that are not 16-byte aligned cost `ragged` more.
     struct Model {
         int tile;
         double lat, w, fixed, fixed_split, ragged;
@@ -384,6 +387,7 @@ cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const flo
                                         {32, 58, 19, 6e3, 9e3, 1.7}};
     const bool rows16 = K % 4 == 0 && N % 4 == 0 && ((((uintptr_t)A) | ((uintptr_t)B)) & 15u) == 0;
     const int64_t chunks = (K + kc - 1) / kc;
+    const int64_t sms = std::max<int64_t>(1, (int64_t)(sm_count() / std::max(1.0, beside)));
     int best = 0;
     double least = 0.0;
     for (int i = 0; i < 6; ++i) {
@@ -392,7 +396,7 @@ cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const flo
         const int64_t tm = (M + m.tile - 1) / m.tile, tn = (N + m.tile - 1) / m.tile;
         if (tm > 65535 || (split && (chunks < 2 || chunks > 8))) continue;
         const int64_t blocks = tm * tn * (split ? chunks : 1);
-        const double u = (double)((blocks + sm_count() - 1) / sm_count());
+        const double u = (double)((blocks + sms - 1) / sms);
         const double per_k = std::max(m.lat, u * m.w) * (rows16 ? 1.0 : m.ragged);
         const double cost = per_k * (double)(split ? kc : K) + (split ? m.fixed_split : m.fixed);
         if (i == 0 || cost < least) {

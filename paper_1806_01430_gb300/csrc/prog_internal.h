@@ -105,6 +105,7 @@ struct RunCtx {
     cudaStream_t st;    // stream the GPU work and copies go to
     bool events;        // record per-loop CUDA events (not while capturing a graph)
     bool out_pending = false;  // copies back queued on the third stream, not joined yet
+    double beside = 1.0;       // a GEMM's share of the work on the GPU meanwhile is 1 / beside
 };
 
 // Output b to the host: into `set` if it is small and goes to the library's own mirror, else

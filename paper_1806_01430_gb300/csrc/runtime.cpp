@@ -714,7 +714,7 @@ gao_status run_gpu_loop(RunCtx& R, int li) {
             if (prec == GAO_GEMM_FP32_SIMT) {
                 if (k0) GAO_CUDA_TRY(record_timing(k0, st));
                 e = launch_gemm_simt(dptr(L.outs[0]), dptr(L.ins[0]), dptr(L.ins[1]), c0 ? c0 : dptr(L.outs[0]),
-                                     A.rows, B.cols, A.cols, (float)L.alpha, beta, p->opts.kchunk, st);
+                                     A.rows, B.cols, A.cols, (float)L.alpha, beta, p->opts.kchunk, st, R.beside);
                 nl += A.rows * B.cols > 0;
                 if (e == cudaSuccess && k1) GAO_CUDA_TRY(record_timing(k1, st));
             } else {
