@@ -110,6 +110,7 @@ struct RunCtx {
 
 // Output b to the host: into `set` if it is small and goes to the library's own mirror, else
 // a copy now.  send_small launches the set and empties it; with d_err, the error word goes along.
+bool sent_small(const BufState& B);
 gao_status output_to_host(RunCtx& R, int b, HostCopySet& set, gao_loop_stat& stat);
 gao_status send_small(HostCopySet& set, cudaStream_t st, const int* d_err = nullptr, int* h_err = nullptr);
 gao_status make_valid(RunCtx& R, int b, bool on_gpu, gao_loop_stat& stat);

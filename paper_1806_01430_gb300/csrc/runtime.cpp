@@ -627,11 +627,14 @@ gao_status send_small(HostCopySet& set, cudaStream_t st, const int* d_err, int* 
     return GAO_OK;
 }
 
+bool sent_small(const BufState& B) {
+    return B.vd && B.host == B.own_host && B.bytes > 0 && B.bytes <= kHostCopyBytes && B.bytes % 4 == 0;
+}
+
 gao_status output_to_host(RunCtx& R, int b, HostCopySet& set, gao_loop_stat& stat) {
     BufState& B = R.p->bufs[(size_t)b];
     if (B.vh) return GAO_OK;
-    if (!B.vd || B.host != B.own_host || B.bytes == 0 || B.bytes > kHostCopyBytes || B.bytes % 4 != 0)
-        return make_valid(R, b, false, stat);
+    if (!sent_small(B)) return make_valid(R, b, false, stat);
     if (set.n == kMaxHostCopies) {
         const gao_status s = send_small(set, R.st);
         if (s != GAO_OK) return s;
@@ -2005,19 +2008,28 @@ gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags)
         if (R.deadline > 0.0 && now_s() > R.deadline) R.timed_out = true;
         if (R.timed_out) break;
     }
+    // small outputs and the error word first, by a kernel right behind the loops', then the others by
+    // the copy engine: the stream goes from kernels to copies once
     HostCopySet small;
     small.n = 0;
-    if (status == GAO_OK && !R.timed_out && !(flags & GAO_RUN_KEEP_DEVICE)) {
-        gao_loop_stat dummy{};
-        for (size_t b = 0; b < p->bufs.size(); ++b)
-            if (p->bufs[b].d.role == GAO_BUF_OUTPUT && !p->bufs[b].vh)
-                if ((status = output_to_host(R, (int)b, small, dummy)) != GAO_OK) break;
-        if (!p->stats.empty()) p->stats.back().d2h_bytes += dummy.d2h_bytes;
-    }
+    const bool back = status == GAO_OK && !R.timed_out && !(flags & GAO_RUN_KEEP_DEVICE);
+    gao_loop_stat dummy{};
+    std::vector<int> large;
+    if (back)
+        for (size_t b = 0; b < p->bufs.size(); ++b) {
+            if (p->bufs[b].d.role != GAO_BUF_OUTPUT || p->bufs[b].vh) continue;
+            if (!sent_small(p->bufs[b])) large.push_back((int)b);
+            else if ((status = output_to_host(R, (int)b, small, dummy)) != GAO_OK) break;
+        }
     if (uses_gpu) {
-        gao_status es = join_outputs(R);
+        const gao_status es = send_small(small, p->st, (const int*)d_err, p->h_err);
         if (es != GAO_OK && status == GAO_OK) status = es;
-        es = send_small(small, p->st, (const int*)d_err, p->h_err);
+    }
+    for (int b : large)
+        if (status == GAO_OK) status = make_valid(R, b, false, dummy);
+    if (back && !p->stats.empty()) p->stats.back().d2h_bytes += dummy.d2h_bytes;
+    if (uses_gpu) {
+        const gao_status es = join_outputs(R);
         if (es != GAO_OK && status == GAO_OK) status = es;
     }
     return status;
