@@ -279,7 +279,8 @@ gao_status make_chain(gao_batch* b, Replica& R, uint64_t mask, const Chain& ch, 
         int64_t M, N, K;
         gemm_shape(p, b->gemm_loop, &M, &N, &K);
         int nl = 0;
-        e = tc_finalize_chain(b->prec, M, N, K, p->arena + p->lay.tc_off, fz[j], b->wide_chains, b->side[j % kSide], &nl);
+        e = tc_finalize_chain(b->prec, M, N, K, p->arena + p->lay.tc_off, fz[j], b->wide_chains,
+                              b->side[j % kSide], &nl);
         cv->kernels += nl;
     }
     if (e == cudaSuccess) e = join_side(b);

@@ -121,7 +121,10 @@ struct HostCopy {
     uint32_t words;  // of 4 bytes
 };
 constexpr int kMaxHostCopies = 128;
-constexpr size_t kHostCopyBytes = 512u << 10;  // largest buffer copied this way
+// Largest buffer copied this way (outputs of one size, us a run, this way / by the copy engine: one of
+// 32 KB 13 / 17, of 512 KB 16 / 20, twelve 53 / 83; the gain then falls to 7 % at 4 MB, and the copy
+// engine leaves the SMs to others).
+constexpr size_t kHostCopyBytes = 512u << 10;
 struct HostCopySet {
     int n;
     HostCopy c[kMaxHostCopies];
@@ -288,13 +291,14 @@ cudaError_t launch_gemm_tc(int prec, float* C, const float* A, const float* B, c
                            int64_t N, int64_t K, float alpha, float beta, int kchunk, int tile_cfg, void* scratch,
                            size_t scratch_bytes, int* err, cudaStream_t st, TcEvents& ev, std::string* why,
                            const TcFuse* fuse = nullptr, const TcPart* part = nullptr, unsigned ready = 0);
-// The bfloat16 planes (FP8: e4m3 codes and scales) of operand `which` (0: A, M x K; 1: B, K x N) of that GEMM (same
-// precision, shapes, K chunk and tile configuration; chain: with `fuse`), formed in its scratch straight from the
+// The bfloat16 planes (FP8: e4m3 codes and scales) of operand `which` (0: A, M x K; 1: B, K x N) of
+// that GEMM (same precision, shapes, K chunk and tile configuration; chain: with `fuse`), formed in
+// its scratch straight from the
 // INIT loop's counter hash of buffer `buf` (times 2^e of each row where rowexp is set), with
 // the values, splitting and zero padding of INIT followed by the GEMM's own split.
 cudaError_t tc_init_planes(int prec, int which, int64_t M, int64_t N, int64_t K, int kchunk, int tile_cfg,
-                           bool chain, uint64_t seed, uint32_t buf, const int8_t* rowexp, void* scratch, size_t scratch_bytes,
-                           cudaStream_t st, int* launches);
+                           bool chain, uint64_t seed, uint32_t buf, const int8_t* rowexp, void* scratch,
+                           size_t scratch_bytes, cudaStream_t st, int* launches);
 
 // Freivalds residual check of C = alpha A B + beta C0 in binary64 (C0 may be null):
 // kernels on st; the residual vectors go to rvec (M) / svec (N) when set; *norms_dev

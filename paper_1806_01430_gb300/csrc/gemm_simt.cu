@@ -18,9 +18,9 @@
 // large tiles, where rows are not 16-byte aligned, through registers (RAG).
 // A small problem has too few tiles to fill the GPU; since the chunks are summed apart anyway, a
 // cluster can split them (no order changes), and smaller tiles serve where that is not enough.
-// Measured, n x n x n, us (before: 128 x 128 tiles of 8 x 8 per thread, scalar FFMAs):
-//   n = 256: 40.8 -> 9.5, 1000: 148 -> 58, 1001: 158 -> 77, 2048: 431 -> 347, 4096: 3020 -> 2500
-//   (55 of 80 TFLOP/s).  What is left: two warps per scheduler issue a packed multiply-add every
+// Measured, n x n x n, us between events (before: 128 x 128 tiles of 8 x 8 per thread, scalar FFMAs):
+//   n = 256: 45 -> 13, 1000: 148 -> 62, 1001: 156 -> 69, 2048: 432 -> 350, 2049: 485 -> 465, 4096: 3028 ->
+//   2490 (55 of 80 TFLOP/s).  What is left: two warps per scheduler issue a packed multiply-add every
 //   other clock with little to cover the operand reads, and the last wave of tiles.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -374,10 +374,11 @@ cudaError_t launch_gemm_simt(float* C, const float* A, const float* B, const flo
     // estimated time: the fullest SM holds u blocks, which take max(lat, u w) clocks per element
     // of K (lat: a block alone, bound by latency; w: its share of a busy SM), plus a fixed cost
     // (launch, first loads, a split's exchange).  The figures are fits to times measured over
-    // n = 128 .. 4096 (within 10 %); a GEMM that shares the GPU with others' is taken to have its
-    // part of the SMs, since the small tiles' extra loads then cost all of them (whole batches, us, as if
-    // alone / so / 128 x 128 tiles of 256 threads for all: 20 programs of 100 to 2000 rows, unaligned,
-    // 1930 / 1847 / 1790, aligned 1532 / 1519 / 1622; eight of 512 to 1024 494 / 428 / 475); rows that are not 16-byte aligned cost `ragged` more.
+    // n = 128 .. 4096 (within 10 %); rows that are not 16-byte aligned cost `ragged` more.  A GEMM
+    // that shares the GPU with others' is taken to have its part of the SMs, since the small tiles'
+    // extra loads then cost all of them (whole batches, us, as if alone / so / 128 x 128 tiles of 256
+    // threads for all: 20 programs of 100 to 2000 rows, unaligned, 1930 / 1847 / 1790, aligned 1532 /
+    // 1519 / 1622; eight of 512 to 1024, unaligned, 494 / 428 / 475).
     struct Model {
         int tile;
         double lat, w, fixed, fixed_split, ragged;

@@ -1037,7 +1037,8 @@ __device__ __forceinline__ void gemm_tc_persistent(const Src& src, int total_til
                 if (ok) {
 #pragma unroll
                     for (int g = 0; g < G; ++g)
-                        store_staged32<EW, !FP8, ANYROW>(ep, row0, (int64_t)n0 + colbase + g * 32, sum + g * 32, stg, lane, &sq);
+                        store_staged32<EW, !FP8, ANYROW>(ep, row0, (int64_t)n0 + colbase + g * 32, sum + g * 32, stg,
+                                                         lane, &sq);
                 }
             }
             if (ep.fuse && ok) {  // fixed butterfly over the warp's rows, one partial per warp
@@ -1405,10 +1406,12 @@ __device__ __forceinline__ void init_gen(const InitSrc& g, uint64_t idx0, float 
 // warp takes four (row, K block) pieces, eight lanes each, lane l of them the quads l, l + 8,
 // l + 16 and l + 24 of its block's 32: the index, the maximum's exchange and the exponent are then
 // paid once for sixteen elements.  With a warp per piece they made the pass issue-bound
-// (3000 x 4100 formed from the hash: 29.2 -> 19.4 us).
+// (3000 x 4100 formed from the hash: 29.2 -> 19.4 us).  Operands kept as binary32, A and B together, us,
+// before and after this and the columns' kernel: 1000^3 16 -> 12, 3000 x 5003 x 4100 80 -> 45, 8192^3
+// 260 -> 127.
 template <bool GEN>
-__global__ void __launch_bounds__(256) quant_rows_fp8_kernel(const float* __restrict__ A, InitSrc gen, int64_t M, int64_t K,
-                                                             int64_t Mp, int64_t Kp, uint8_t* __restrict__ q,
+__global__ void __launch_bounds__(256) quant_rows_fp8_kernel(const float* __restrict__ A, InitSrc gen, int64_t M,
+                                                             int64_t K, int64_t Mp, int64_t Kp, uint8_t* __restrict__ q,
                                                              uint8_t* __restrict__ sfa) {
     const int lane = threadIdx.x & 31, l8 = lane & 7;
     const int64_t kbs = Kp / 128;
@@ -1465,12 +1468,13 @@ __global__ void __launch_bounds__(256) quant_rows_fp8_kernel(const float* __rest
 // bytes]; CTA = (K block, 64 columns).  A warp reads 32 consecutive columns of a row a word
 // each, so rows of any alignment load whole lines; all 32 of a thread's loads are in flight.
 // Columns are packed lane per column (no bank conflicts) and go out through a byte tile as
-// whole 128-byte rows of q^T.  HBM-bound: 4100 x 5003 in 20.7 us = 5.0 TB/s; 48.1
-// with a row's load waited for at a time and a column's packing lanes in conflict on its banks.
+// whole 128-byte rows of q^T.  Reading binary32 it is HBM-bound: 4100 x 5003 in 20.7 us = 5.0 TB/s;
+// 48.1 with a row's load waited for at a time and a column's packing lanes in conflict on its
+// banks.  Forming the values from the hash (GEN) it is bound by integer issue: 27 us.
 constexpr int kQuantCols = 64;
 template <bool GEN>
-__global__ void __launch_bounds__(256) quant_cols_fp8_kernel(const float* __restrict__ B, InitSrc gen, int64_t K, int64_t N,
-                                                             int64_t Np, int64_t Kp, uint8_t* __restrict__ q,
+__global__ void __launch_bounds__(256) quant_cols_fp8_kernel(const float* __restrict__ B, InitSrc gen, int64_t K,
+                                                             int64_t N, int64_t Np, int64_t Kp, uint8_t* __restrict__ q,
                                                              uint8_t* __restrict__ sfb) {
     __shared__ __align__(16) float tile[128][kQuantCols + 1];
     constexpr int kRed = GEN ? 8 : 4;
@@ -1794,9 +1798,12 @@ struct TcShape {
 // 5000^3 1034 -> 997; 2 to 5% also back to back, at the power cap.  Outside: fewer tiles leave
 // too few 256-row ones to go round (3001 x 1500 x 3003, three terms 162 -> 166); shorter inner
 // dimensions are bound by the epilogue, which a pair's two CTAs run in step (two terms 6000 x
-// 1100 x 6000 240 -> 242, 4001 x 500 x 3003 60 -> 78); larger planes leave nothing to find in L2
-// (8192^3 without a chain, three terms 3761 -> 4091).  Without a chain a pair is up to 6% faster
-// alone, but 1 to 4% slower back to back, where power bounds it.
+// 1100 x 6000 240 -> 242, 4001 x 500 x 3003 60 -> 78).  In between, 6000 x K x 6000: two terms K = 1280
+// 252 -> 252, 1400 272 -> 268, 1450 288 -> 277; three terms gain 2 to 4% from K = 1000 on there, but
+// nothing at 4096 x K x 4096 up to 1500 (242 -> 242): the line stands where both terms have gained.
+// Larger planes leave nothing to find in L2 (8192^3 without a chain, three terms 3761 -> 4091).
+// Without a chain a pair is up to 6% faster alone, but 1 to 4% slower back to back, where power
+// bounds it.
 bool tc_split_default(int planes, bool chain, int64_t M, int64_t N, int64_t K, int tile_cfg) {
     return planes > 1 && chain && (tile_cfg & 15) == 0 && K >= 1500 &&
            ((M + BM - 1) / BM) * ((N + 127) / 128) >= 6 * (int64_t)sm_count() &&
@@ -1837,8 +1844,8 @@ TcShape tc_shape(int prec, int64_t M, int64_t Mlay, int64_t N, int64_t K, int kc
 }  // namespace
 
 cudaError_t tc_init_planes(int prec, int which, int64_t M, int64_t N, int64_t K, int kchunk, int tile_cfg,
-                           bool chain, uint64_t seed, uint32_t buf, const int8_t* rowexp, void* scratch, size_t scratch_bytes,
-                           cudaStream_t st, int* launches) {
+                           bool chain, uint64_t seed, uint32_t buf, const int8_t* rowexp, void* scratch,
+                           size_t scratch_bytes, cudaStream_t st, int* launches) {
     *launches = 0;
     if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_FP8 || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
     if (tc_scratch_bytes(prec, M, N, K) > scratch_bytes || ((uintptr_t)scratch & 1023u)) return cudaErrorInvalidValue;

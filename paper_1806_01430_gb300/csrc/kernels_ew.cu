@@ -256,7 +256,8 @@ __global__ void __launch_bounds__(kThreads) host_copies_kernel(const __grid_cons
 // selects, and forming all three operations, cost ten instructions a value and made the pass
 // issue-bound.
 template <int N>
-__device__ __forceinline__ void chain_axpy(float alpha, float (&cur)[N][4], const float (&x)[N][4], const float (&y)[N][4]) {
+__device__ __forceinline__ void chain_axpy(float alpha, float (&cur)[N][4], const float (&x)[N][4],
+                                           const float (&y)[N][4]) {
 #pragma unroll
     for (int k = 0; k < N; ++k)
 #pragma unroll
@@ -1133,7 +1134,8 @@ __device__ __forceinline__ void edge_store(float* row, int64_t c0, int64_t cols,
 #pragma unroll
         for (int k = 0; k < 2; ++k)
             if (out.has<VEC>(4 * k))
-                *reinterpret_cast<float4*>(row + c0 + 4 * k) = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+                *reinterpret_cast<float4*>(row + c0 + 4 * k) =
+                    make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
     } else {
         const int lane = threadIdx.x & 31;
         __syncwarp();  // the previous row's reads are done
@@ -1233,8 +1235,8 @@ __global__ void __launch_bounds__(kStencilThreads, edge_blocks(STORE))
     const float* pn = row_ptr(r0 + 5);
     // output row `row`: raw rows row, row + 1 in x0, x1 and B's rows row - 1, row in b0, b1; raw
     // row + 2 goes to x2 and B's row + 1 to b2
-    auto step = [&](int64_t row, EdgeRow& next, const EdgePairs& x0, const EdgePairs& x1, EdgePairs& x2, const EdgePairs& b0,
-                    const EdgePairs& b1, EdgePairs& b2) {
+    auto step = [&](int64_t row, EdgeRow& next, const EdgePairs& x0, const EdgePairs& x1, EdgePairs& x2,
+                    const EdgePairs& b0, const EdgePairs& b1, EdgePairs& b2) {
         edge_pairs(x2, next);
         edge_load<VEC>(next, pn, row + 5 < ylim, inc);
         pn += cols;

@@ -94,7 +94,10 @@ namespace gao {
 constexpr int kMaxRowBlocks = 4;                 // row blocks of an overlapped GEMM loop
 constexpr int kMaxColParts = 2;                  // column ranges of its first row block
 constexpr size_t kPipelineMinBytes = 16u << 20;  // smallest A worth overlapping
-constexpr size_t kPlanesMinBytes = 16u << 20;    // smallest operand of a GEMM with its chain formed as planes
+// Smallest operand of a GEMM with its chain formed as planes.  Below it the split saved and the
+// operand's own INIT launch nearly cancel (six-loop pass, us, kept binary32 / planes, two and three
+// terms: n = 512 43 / 40, 51 / 49; 1024 51 / 51, 62 / 63; 1536 63 / 62, 76 / 75; 4096 664 / 643).
+constexpr size_t kPlanesMinBytes = 16u << 20;
 
 // One execution of a program (or of a batch of programs sharing a stream).
 struct RunCtx {

@@ -1610,21 +1610,18 @@ double ev_ms(cudaEvent_t a, cudaEvent_t b) {
 }
 }  // namespace
 
-// Everything a run under a gene puts on the program's stream, in program order, with the
-// host loops run in between: residency reset, the error word, each loop's copies and
-// kernels (or its host loop), the outputs' copies back and the error word's read-back.
-// When every loop is on the GPU this is also what a CUDA graph of the run captures.
 // The GEMM loop that alone reads INIT loop li's output b, as its A (*which = 0) or its B
 // (*which = 1), when that GEMM runs on the tensor cores: b is then formed straight into the
 // GEMM's bfloat16 planes or e4m3 codes, never as binary32.  A GEMM with its chain takes operands of
-// at least kPlanesMinBytes this way; below that the split it saves is a few us.  Whole pass:
+// at least kPlanesMinBytes this way (see there).  Whole pass:
 // six-loop program 4096, three terms, B: 664 -> 643 us; twelve-loop 6000, K = 1500, two terms, A
 // and B: 455 -> 435.  -1 otherwise (b is not a TEMP buffer, is read by anything else or written
 // by another loop, the caller holds its device pointer, the GEMM reads it twice or also as C0,
 // another GEMM on the GPU uses the one room for planes, transfers are per loop).
 int planes_consumer(const gao_prog* p, int li, int b, uint64_t gene_mask, bool fuse, int* which) {
     const BufState& B = p->bufs[(size_t)b];
-    if (B.d.role != GAO_BUF_TEMP || B.held || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT || p->lay.tc_bytes == 0) return -1;
+    if (B.d.role != GAO_BUF_TEMP || B.held || p->opts.transfer_mode != GAO_TRANSFER_RESIDENT || p->lay.tc_bytes == 0)
+        return -1;
     const int prec = p->opts.gemm_prec;
     if (prec < GAO_GEMM_BF16 || prec > GAO_GEMM_FP8) return -1;
     int reader = -1, gemms = 0;
@@ -1697,14 +1694,19 @@ gao_status run_gpu_init_planes(RunCtx& R, int li, const int* cons, const int* wh
         const int rs = (int)((L.flags >> t) & 1);
         int l = 0;
         Chain ch;
+        const bool chain = find_chain(p, cons[t], p->run_mask, p->run_fuse, &ch);
         GAO_CUDA_TRY(tc_init_planes(p->opts.gemm_prec, wh[t], A.rows, Bm.cols, A.cols, p->opts.kchunk,
-                                    p->opts.tile_cfg, find_chain(p, cons[t], p->run_mask, p->run_fuse, &ch), p->opts.seed, (uint32_t)L.outs[t], rs ? set.rowexp : nullptr,
-                                    a + p->lay.tc_off, p->lay.tc_bytes, st, &l));
+                                    p->opts.tile_cfg, chain, p->opts.seed, (uint32_t)L.outs[t],
+                                    rs ? set.rowexp : nullptr, a + p->lay.tc_off, p->lay.tc_bytes, st, &l));
         nl += l;
     }
     return GAO_OK;
 }
 
+// Everything a run under a gene puts on the program's stream, in program order, with the
+// host loops run in between: residency reset, the error word, each loop's copies and
+// kernels (or its host loop), the outputs' copies back and the error word's read-back.
+// When every loop is on the GPU this is also what a CUDA graph of the run captures.
 gao_status enqueue_run(RunCtx& R, uint64_t gene_mask, bool fuse, uint32_t flags) {
     gao_prog* p = R.p;
     const int n = (int)p->loops.size();
