@@ -1068,34 +1068,40 @@ struct EdgeRow {
     float4 g[2];
 };
 
-// Which of a lane's eight columns: the first n (with 16-byte rows none, four or eight: two flags that
-// stay in predicates; else a count, where eight flags would not).
+// Which of a lane's eight columns c0 .. c0 + 7 lie inside the image (none unless `mine`): with 16-byte
+// rows none, the first four or all, two flags that stay in predicates; else a count, where eight
+// flags would not.
+template <bool VEC>
 struct EdgeCols {
-    int n;
     bool lo, hi;
-    __device__ __forceinline__ explicit EdgeCols(int count) : n(count), lo(count > 0), hi(count > 4) {}
-    template <bool VEC>
-    __device__ __forceinline__ bool has(int q) const {
-        return VEC ? (q < 4 ? lo : hi) : q < n;
-    }
+    __device__ __forceinline__ EdgeCols(int64_t c0, int64_t cols, bool mine)
+        : lo(mine && c0 >= 0 && c0 < cols), hi(mine && c0 >= 0 && c0 + 4 < cols) {}
+    __device__ __forceinline__ bool has(int q) const { return q < 4 ? lo : hi; }
+};
+template <>
+struct EdgeCols<false> {
+    int n;
+    __device__ __forceinline__ EdgeCols(int64_t c0, int64_t cols, bool mine)
+        : n(!mine || c0 < 0 || c0 >= cols ? 0 : cols - c0 < kEdgeNC ? (int)(cols - c0) : kEdgeNC) {}
+    __device__ __forceinline__ bool has(int q) const { return q < n; }
 };
 
 // p: row y's first column of the lane (any value when the row is outside the image).
 template <bool VEC>
 __device__ __forceinline__ void edge_load(EdgeRow& r, const float* __restrict__ p, bool row_in,
-                                          const EdgeCols& in) {
+                                          const EdgeCols<VEC>& in) {
     r.g[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     r.g[1] = r.g[0];
     if (!row_in) return;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         if (VEC) {
-            if (in.has<VEC>(4 * k)) r.g[k] = __ldg(reinterpret_cast<const float4*>(p + 4 * k));
+            if (in.has(4 * k)) r.g[k] = __ldg(reinterpret_cast<const float4*>(p + 4 * k));
         } else {
-            if (in.has<VEC>(4 * k)) r.g[k].x = __ldg(p + 4 * k);
-            if (in.has<VEC>(4 * k + 1)) r.g[k].y = __ldg(p + 4 * k + 1);
-            if (in.has<VEC>(4 * k + 2)) r.g[k].z = __ldg(p + 4 * k + 2);
-            if (in.has<VEC>(4 * k + 3)) r.g[k].w = __ldg(p + 4 * k + 3);
+            if (in.has(4 * k)) r.g[k].x = __ldg(p + 4 * k);
+            if (in.has(4 * k + 1)) r.g[k].y = __ldg(p + 4 * k + 1);
+            if (in.has(4 * k + 2)) r.g[k].z = __ldg(p + 4 * k + 2);
+            if (in.has(4 * k + 3)) r.g[k].w = __ldg(p + 4 * k + 3);
         }
     }
 }
@@ -1121,7 +1127,7 @@ __device__ __forceinline__ void edge_pairs(EdgePairs& r, const EdgeRow& v) {
 // 32 consecutive columns and not a word every 32 bytes (pass, us: 4095 x 4097 with its magnitude
 // written 109 -> 70, 2000 x 2001 with three of its maps 81.5 -> 36.4).
 template <bool VEC>
-__device__ __forceinline__ void edge_store(float* row, int64_t c0, int64_t cols, const EdgeCols& out, const f32x2 v[4],
+__device__ __forceinline__ void edge_store(float* row, int64_t c0, int64_t cols, const EdgeCols<VEC>& out, const f32x2 v[4],
                                            float* stage) {
     float x[kEdgeNC];
 #pragma unroll
@@ -1133,7 +1139,7 @@ __device__ __forceinline__ void edge_store(float* row, int64_t c0, int64_t cols,
     if (VEC) {
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if (out.has<VEC>(4 * k))
+            if (out.has(4 * k))
                 *reinterpret_cast<float4*>(row + c0 + 4 * k) =
                     make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
     } else {
@@ -1185,15 +1191,14 @@ __global__ void __launch_bounds__(kStencilThreads, edge_blocks(STORE))
     float* stage = s_stage[threadIdx.x >> 5];
     const int64_t c0 = ((int64_t)blockIdx.x * (kStencilThreads / 32) + (threadIdx.x >> 5)) * kEdgeCols - NC + NC * lane;
     // this lane's columns inside the image, and those it produces
-    const EdgeCols inc(c0 < 0 || c0 >= cols ? 0 : cols - c0 < NC ? (int)(cols - c0) : NC);
-    const EdgeCols outc(lane >= 1 && lane <= 30 ? inc.n : 0);
+    const EdgeCols<VEC> inc(c0, cols, true), outc(c0, cols, lane >= 1 && lane <= 30);
     // output rows [r0, r1) of this block's strip; raw rows r0 - 2 .. r1 + 1 are read
     const int64_t r0 = row_begin + (int64_t)blockIdx.y * strip;
     const int64_t r1 = r0 + strip < row_end ? r0 + strip : row_end;
     const int64_t ylim = r1 + 2 < rows ? r1 + 2 : rows;
     // a lane whose columns are all inside the image zeroes none of its B values but in the
     // rows above and below it, so it skips the per-value choice elsewhere
-    const bool all_in = inc.n == NC;
+    const bool all_in = inc.has(0) && inc.has(NC - 1);
     // B's row from the raw rows above, at and below it (zero outside the image)
     auto blur = [&](EdgePairs& b, const EdgePairs& xu, const EdgePairs& xm, const EdgePairs& xd, bool row_in) {
 #pragma unroll
@@ -1202,7 +1207,7 @@ __global__ void __launch_bounds__(kStencilThreads, edge_blocks(STORE))
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float2 u = unpack2(b.p[k + 1]);
-                b.p[k + 1] = pack2(row_in && inc.has<VEC>(k) ? u.x : 0.0f, row_in && inc.has<VEC>(k + 4) ? u.y : 0.0f);
+                b.p[k + 1] = pack2(row_in && inc.has(k) ? u.x : 0.0f, row_in && inc.has(k + 4) ? u.y : 0.0f);
             }
         }
     };
@@ -1280,10 +1285,10 @@ __global__ void __launch_bounds__(kStencilThreads, edge_blocks(STORE))
                 float t;
                 if (VEC) {
                     const float2 g = unpack2(add2(add2(m[0], m[1]), add2(m[2], m[3])));
-                    t = g.x + (inc.hi ? g.y : 0.0f);
+                    t = g.x + (inc.has(4) ? g.y : 0.0f);
                 } else {
 #pragma unroll
-                    for (int q = 0; q < NC; ++q) v[q] = outc.has<VEC>(q) ? v[q] : 0.0f;
+                    for (int q = 0; q < NC; ++q) v[q] = outc.has(q) ? v[q] : 0.0f;
                     t = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
                 }
                 comp_add(rs, rc, t);
@@ -1301,11 +1306,11 @@ __global__ void __launch_bounds__(kStencilThreads, edge_blocks(STORE))
         if (out.keys && r1 > r0) {
 #pragma unroll
             for (int q = 0; q < NC; ++q)
-                if (outc.has<VEC>(q)) atomicMax(out.keys + c0 + q, mk[q]);  // max: exact and order-free
+                if (outc.has(q)) atomicMax(out.keys + c0 + q, mk[q]);  // max: exact and order-free
         }
         if (out.part) {
             __shared__ double wsum[kStencilThreads / 32];
-            double acc = (!VEC || outc.lo) ? (double)rs + (double)rc : 0.0;
+            double acc = (!VEC || outc.has(0)) ? (double)rs + (double)rc : 0.0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (lane == 0) wsum[threadIdx.x >> 5] = acc;
